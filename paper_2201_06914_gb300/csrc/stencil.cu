@@ -95,9 +95,12 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
     float *dbring = uring + NU * S::USLOT;
     __shared__ float sq[TY][TX];
     __shared__ int inj_lo, inj_hi;
+    __shared__ step::f2 coef[8];
 
     const int ntx = (G.NX + TX - 1) / TX, nty = (G.NY + TY - 1) / TY;
     const int ntiles = ntx * nty * ((G.NZ + G.tz - 1) / G.tz);
+    pdl_trigger();
+    pdl_wait();
     if ((int)blockIdx.x >= ntiles) {
         gather_rows(A, blockIdx.x - ntiles);
         return;
@@ -185,6 +188,7 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
     if (tid == 0) {
         inj_lo = 1 << 30;
         inj_hi = -1;
+        step::coef_store(&coef, G);
     }
     __syncthreads();
     if (tile_inj)
@@ -221,6 +225,7 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
     cp_async_wait<LA - 1>();
     __syncthreads();
     const int zlo = inj_lo, zhi = inj_hi;
+    const step::Coef K = step::coef_load(&coef);
 #pragma unroll
     for (int k = 0; k < RAD; k++) win[RAD + k] = (z0 + k < G.NZ) ? step::lds(ub + (uint32_t)k * USZ) : step::zero();
 
@@ -277,7 +282,7 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
             P4 dn, un;
             float sdv[4];
             step::step4<(TY > 1), WD>(&win[ph], yp, ym, wl, wr, din, bb, &sq[ly][4 * lx], inj,
-                                  col_int && z >= zs0 && z < zs1, sdx, z, G, dn, un, sdv);
+                                  col_int && z >= zs0 && z < zs1, sdx, z, G, K, dn, un, sdv);
             if (has_pad) step::zero_pad(xc, G.NX, dn, un);   // padding columns stay zero
             const long long oz = (long long)z * PS;
             *(P4 *)(uo + oz) = un;
@@ -319,7 +324,7 @@ static void launch_variant(const GridDev &G, const StencilArgs &A, dim3 grid, cu
 {
     using S = StencilShape<TXT, TY, stencil_na<TXT, TY, IMG>()>;
     cudaFuncSetAttribute(stencil_kernel<TXT, TY, IMG, WD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    stencil_kernel<TXT, TY, IMG, WD><<<grid, S::NT, S::SMEM, s>>>(G, A);
+    pdl_launch(stencil_kernel<TXT, TY, IMG, WD>, grid, S::NT, S::SMEM, s, G, A);
 }
 
 template <int TXT, int TY>

@@ -17,7 +17,25 @@
 // neighbouring segments by 8 planes of stage-A work: the halo of step 2 is recomputed
 // rather than exchanged.  Stage B trails stage A by 4 planes: u^{n+1} of the own float4
 // lives in a register window, its x neighbours in a shared ring of 8 planes, and d^{n+1}
-// replaces d^n in the increment ring slot it came from.
+// replaces d^n in the ring slot it came from.
+//
+// What bounds it: a plane of the march is one long chain of instructions per warp (12 warps a
+// SM, all the registers and shared memory allow), so its time is the number of instructions
+// times their latency, as long as the loop stays in the instruction cache.  Hence
+//   - every shared-memory access has a constant offset from one of two registers (rings of two
+//     groups of four planes) and every global one is one multiply-add away from one offset;
+//   - nothing outside the grid is tested: staging zero-fills it, and dt^2/m = 0 there makes both
+//     steps give zero; the absorbing layer is a branch of the whole warp;
+//   - the constants stay in registers (stencil_step.cuh), and groups without injection entries
+//     run a copy of the loop without the lookups;
+//   - the loop is unrolled by four planes: 185 instructions a warp and plane in 13 KB.  By three
+//     it needs ring arithmetic (374 instructions a plane, 18 KB); by eight it drops the moves of
+//     the register windows but stalls on instruction fetch (27 KB: 270 us where four planes take
+//     218 and three took 300).
+// Measured per launch of the 1601 x 401 model (padded 1681 x 481): 64 shots 218 us (300 before;
+// 4.75 TB/s of the 20 B per point and shot it must move), 32 shots 121 (167), 16 shots 68 (94.5),
+// 8 shots 41 (57), one shot 15 (33); with the imaging condition, 16 shots: 116 us (150 before,
+// 130 without the L2 prefetch); one shot of 201 x 201: 11.2 us (39).
 //
 // Injection uses a CSR table keyed by (tile, plane of the extended segment) that lists
 // every entry inside the extended tile (points in an overlap appear in both tiles);
@@ -28,51 +46,49 @@
 // was a pair, the row of its first step as R (u^{n-1} + d^n) from the input of that launch
 // and the stored increment, the same addition stage A made.
 #include <cstdlib>
+#include <type_traits>
 
 #include "stencil_step.cuh"
 
 namespace wp {
 
 using step::P4;
+using step::f2;
 
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-#ifndef WP_STENCIL2_U
-#define WP_STENCIL2_U 3
-#endif
 template <int TXT>
 struct Stencil2Shape {
     static constexpr int TX = 4 * TXT;
     static constexpr int C = TX - 2 * RAD;          // core columns (stage B)
     static constexpr int NT = TXT;
     static constexpr int W = TX + 2 * RAD;          // u ring row (x halos of stage A)
-    static constexpr int U = WP_STENCIL2_U;         // planes per unrolled group
+    static constexpr int U = 4;                     // planes per unrolled group
+    static constexpr int NR = 8;                    // ring slots (two groups)
     static constexpr int LA = 3;                    // planes in flight
-    static constexpr int NU = 8;                    // u^n ring: planes z .. z+4+LA
-    static constexpr int NDB = 8;                   // d/b ring: planes z-4 .. z+LA
-    static constexpr int NV = 8;                    // u^{n+1} ring: planes z-4 .. z
-    static constexpr int UCH = W / 4, DBCH = 2 * TX / 4;
-    static constexpr int UK = (UCH + NT - 1) / NT, DK = (DBCH + NT - 1) / NT;
-    static constexpr size_t SMEM = (size_t)(NU * W + NDB * 2 * TX + NV * TX) * sizeof(float);
-    static constexpr int MINB = 8192 / (NT * 24) > 16 ? 16 : 8192 / (NT * 24);
-    static_assert(RAD + 1 + LA <= NU && LA + RAD + 1 <= NDB && RAD + 1 <= NV, "rings");
+    static constexpr int SLOT = W + 3 * TX;         // u^n row with halos, increment, dt^2/m, u^{n+1}
+    // (the last lane reads one float4 past the u^{n+1} ring)
+    static constexpr size_t SMEM = ((size_t)NR * SLOT + 4) * sizeof(float);
+    // 6 blocks of 64 threads (33 KB of rings each) or 12 of 32: registers <= 168
+    static constexpr int MINB = 384 / NT;
+    static_assert(NR == 2 * U && U == RAD && RAD + 1 + LA <= NR, "rings");
 };
 
 template <int TXT, bool WD, bool IMG>
 __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel(const GridDev G, const StencilArgs A)
 {
     using S = Stencil2Shape<TXT>;
-    constexpr int TX = S::TX, C = S::C, W = S::W, NT = S::NT, LA = S::LA, U = S::U;
-    constexpr int NU = S::NU, NDB = S::NDB, NV = S::NV;
-    constexpr uint32_t USZ = W * 4, DSZ = 2 * TX * 4, VSZ = TX * 4;
+    constexpr int TX = S::TX, C = S::C, W = S::W, NT = S::NT, LA = S::LA, NR = S::NR, U = S::U;
+    constexpr uint32_t SL = S::SLOT * 4, OD = W * 4, OB = OD + TX * 4, OV = OB + TX * 4;   // slot bytes, offsets
     extern __shared__ float4 smem4[];
-    float *uring = (float *)smem4;
-    float *dbring = uring + NU * W;
-    float *vring = dbring + NDB * 2 * TX;
     __shared__ float sq[2][TX];   // injected terms [stage][column]
     __shared__ int inj_lo, inj_hi;
+    __shared__ f2 coef[8];
 
     const int ntx = (G.NXp + C - 1) / C;
     const int ntiles = ntx * ((G.NZ + G.tz2 - 1) / G.tz2);
+    pdl_trigger();
+    pdl_wait();
     if ((int)blockIdx.x >= ntiles) {
         gather_rows(A, blockIdx.x - ntiles);
         return;
@@ -81,72 +97,63 @@ __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel
     const long long sh = blockIdx.y;
     const int x0 = (tile % ntx) * C - RAD;
     const int z0 = (tile / ntx) * G.tz2, z1 = min(z0 + G.tz2, G.NZ);
-    const int zs = z0 - RAD, ze = z1 + RAD;   // stage-A planes (outside the grid: zeros)
-    const int KP = G.tz2 + 2 * RAD;           // table keys per tile
+    const int zs = z0 - RAD, nrel = z1 - z0 + 2 * RAD;   // stage-A planes zs .. zs + nrel - 1
+    const int KP = G.tz2 + 2 * RAD;                      // table keys per tile
     const int NXp = G.NXp, NZ = G.NZ;
+    const int xc = x0 + 4 * lx;
+    const bool a_ok = xc >= 0 && xc < NXp;               // the float4 lies inside the field
     const float *__restrict__ u = A.u_in + sh * A.u_in_ss;
 
-    uint32_t us[S::UK];
-    const float *ug[S::UK];
-    int un16[S::UK];
-#pragma unroll
-    for (int k = 0; k < S::UK; k++) {
-        const int c = lx + k * NT;
-        const int x = x0 - RAD + 4 * c;
-        const bool v = c < S::UCH && x >= 0 && x < NXp;
-        un16[k] = v ? 16 : 0;
-        us[k] = (uint32_t)(4 * c) * 4;
-        ug[k] = u + (v ? x : 0);
-    }
-    uint32_t ds[S::DK];
-    const float *dg[S::DK];
-    int dn16[S::DK];
-#pragma unroll
-    for (int k = 0; k < S::DK; k++) {
-        const int c = lx + k * NT;
-        const int a = c / (TX / 4), k4 = c % (TX / 4);
-        const int x = x0 + 4 * k4;
-        const bool v = c < S::DBCH && x >= 0 && x < NXp;
-        dn16[k] = v ? 16 : 0;
-        ds[k] = (uint32_t)(a * TX + 4 * k4) * 4;
-        dg[k] = (a == 1 ? A.b : A.d_in + sh * A.d_in_ss) + (v ? x : 0);
-    }
-    const uint32_t su0 = (uint32_t)__cvta_generic_to_shared(uring);
-    const uint32_t sd0 = (uint32_t)__cvta_generic_to_shared(dbring);
-    const uint32_t sv0 = (uint32_t)__cvta_generic_to_shared(vring);
-    // plane k of u^n into ring slot (k - zs) mod NU; planes outside the grid are not copied
-    // (their slots are never read)
-    auto issue_u = [&](int k) {
-        if (k < 0 || k >= NZ) return;
-        const uint32_t base = su0 + (uint32_t)((k - zs) & (NU - 1)) * USZ;
-        const int ko = k * NXp;
-#pragma unroll
-        for (int q = 0; q < S::UK; q++)
-            if ((q + 1) * NT <= S::UCH || lx + q * NT < S::UCH) cp_async16(base + us[q], ug[q] + ko, un16[q]);
+    // Staging: thread lx copies float4 lx of the u row (x0 - 4 + 4 lx; lanes 0 and 1 also the
+    // two last ones) and its own float4 of the increment and of dt^2/m.  Everything outside
+    // the grid is zero-filled, where dt^2/m = 0 makes both steps give zero: stage A needs no
+    // test for columns or planes beyond the grid.
+    const int xu = x0 - RAD + 4 * lx, xv = xu + TX;
+    const int nu = xu >= 0 && xu < NXp ? 16 : 0, nv = xv < NXp ? 16 : 0, nd = a_ok ? 16 : 0;
+    const int own = a_ok ? xc : 0;
+    // (a copy of zero bytes reads nothing, but its address stays inside the array)
+    const float *gu = u + (nu ? xu : 0), *gv = u + (nv ? xv : 0);
+    const float *gd = A.d_in + sh * A.d_in_ss + own, *gb = A.b + own;
+    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(smem4) + 16u * lx;
+    // Plane zs + r (zeros outside the grid and past the segment) into the slot at `o`; ko: the
+    // plane's offset in floats.  The tests are uniform over the block.
+    const int ulim = min(NZ, z1 + 2 * RAD), dlim = min(NZ, z1 + RAD);
+    auto issue_u = [&](int r, int ko, uint32_t o) {
+        if ((unsigned)(zs + r) < (unsigned)ulim) {
+            cp_async16(o, gu + ko, nu);
+            if (lx < 2) cp_async16(o + TX * 4, gv + ko, nv);
+        } else {
+            step::sts(o, step::zero());
+            if (lx < 2) step::sts(o + TX * 4, step::zero());
+        }
     };
-    auto issue_db = [&](int k) {
-        if (k < 0 || k >= NZ || k >= ze) return;
-        const uint32_t base = sd0 + (uint32_t)((k - zs) & (NDB - 1)) * DSZ;
-        const int ko = k * NXp;
-#pragma unroll
-        for (int q = 0; q < S::DK; q++)
-            if ((q + 1) * NT <= S::DBCH || lx + q * NT < S::DBCH) cp_async16(base + ds[q], dg[q] + ko, dn16[q]);
+    auto issue_db = [&](int r, int ko, uint32_t o) {
+        if ((unsigned)(zs + r) < (unsigned)dlim) {
+            cp_async16(o + OD, gd + ko, nd);
+            cp_async16(o + OB, gb + ko, nd);
+        } else {
+            step::sts(o + OD, step::zero());
+            step::sts(o + OB, step::zero());
+        }
     };
 
+    // group g < LA holds u plane 4 + g and increment plane g; group 0 also u planes 0 .. 3
 #pragma unroll
-    for (int k = 0; k < RAD; k++) issue_u(zs + k);
+    for (int r = 0; r < RAD; r++) issue_u(r, (zs + r) * NXp, sb + r * SL);
 #pragma unroll
     for (int g = 0; g < LA; g++) {
-        issue_u(zs + RAD + g);
-        issue_db(zs + g);
+        issue_u(RAD + g, (zs + RAD + g) * NXp, sb + (RAD + g) * SL);
+        issue_db(g, (zs + g) * NXp, sb + g * SL);
         cp_async_commit();
     }
+
     const int *off = A.inj ? A.inj_off + sh * ((long long)ntiles * KP + 1) : nullptr;
     const long long key0 = (long long)tile * KP;
     const bool tile_inj = off && off[key0] < off[key0 + KP];
     if (lx == 0) {
         inj_lo = 1 << 30;
-        inj_hi = -1;
+        inj_hi = -(1 << 30);
+        step::coef_store(&coef, G);
     }
     __syncthreads();
     if (tile_inj)
@@ -158,72 +165,79 @@ __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel
     const float *trA = tile_inj ? A.traces + sh * A.tr_ss + (long long)A.step * A.tr_ts : nullptr;
     const float *trB = tile_inj ? A.traces + sh * A.tr_ss + (long long)A.step2 * A.tr_ts : nullptr;
 
-    const int xc = x0 + 4 * lx;
-    const bool a_ok = xc >= 0 && xc < NXp;                 // stage-A float4 inside the field
-    const bool core = lx >= 1 && lx <= TXT - 2;            // stage-B lanes
-    const bool b_ok = a_ok && core;
+    const bool st_ok = a_ok && lx >= 1 && lx <= TXT - 2;   // core float4 inside the field: stores
     float sdx[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) sdx[j] = damp_term(xc + j, G.nx, G.nbl, G.hs0x, G.inv_nbl);
-    const bool col_int = sdx[0] == 0.f && sdx[1] == 0.f && sdx[2] == 0.f && sdx[3] == 0.f;
-    const bool has_pad = xc + 4 > G.NX;
-    const long long own = a_ok ? xc : 0;
-    float *uo = A.u_out + sh * A.u_out_ss + own;
-    float *dout = A.d_out + sh * A.d_out_ss + own;
-    float *u1o = A.u1_out ? A.u1_out + sh * A.u1_ss + own : nullptr;
-    float *d1o = A.d1_out ? A.d1_out + sh * A.d1_ss + own : nullptr;
+    // the whole warp outside the x absorbing layers (columns outside the grid do not matter)
+    const bool warp_int =
+        __all_sync(0xffffffffu, !a_ok || (sdx[0] == 0.f && sdx[1] == 0.f && sdx[2] == 0.f && sdx[3] == 0.f));
+    const int ri0 = G.nbl - zs, ri1 = G.nbl + G.nz - zs;   // rel of the planes outside the z layers
+    float *uo = A.u_out + sh * A.u_out_ss + own, *dout = A.d_out + sh * A.d_out_ss + own;
+    float *u1o = IMG ? nullptr : A.u1_out + sh * A.u1_ss + own;
 
-    // wa[i]: u^n of plane zb + i - 4; wb[i]: u^{n+1} of plane zb + i - 8 (group start zb)
+    // Register windows of the own float4, slid by U planes after every group (first plane r0):
+    // wa[i]: u^n of plane zs + r0 - 4 + i; wb[i]: u^{n+1} of plane zs + r0 - 8 + i.
     P4 wa[2 * RAD + U], wb[2 * RAD + U];
-    const P4 zero4 = step::zero();
 #pragma unroll
     for (int k = 0; k < RAD; k++) {
         const int zz = zs - RAD + k;
-        wa[k] = (a_ok && zz >= 0) ? *(const P4 *)(u + (long long)zz * NXp + own) : zero4;
+        wa[k] = (a_ok && zz >= 0) ? *(const P4 *)(u + (long long)zz * NXp + own) : step::zero();
     }
 #pragma unroll
-    for (int k = 0; k < 2 * RAD; k++) wb[k] = zero4;
-    const uint32_t ub = su0 + (uint32_t)(RAD + 4 * lx) * 4;
-    const uint32_t db = sd0 + (uint32_t)(4 * lx) * 4;
-    const uint32_t vb = sv0 + (uint32_t)(4 * lx) * 4;
+    for (int k = 0; k < 2 * RAD; k++) wb[k] = step::zero();
     cp_async_wait<LA - 1>();
     __syncthreads();
     const int klo = inj_lo, khi = inj_hi;
+    const step::Coef K = step::coef_load(&coef);
 #pragma unroll
-    for (int k = 0; k < RAD; k++) {
-        const int zz = zs + k;
-        wa[RAD + k] = (zz >= 0 && zz < NZ) ? step::lds(ub + (uint32_t)k * USZ) : zero4;
-    }
+    for (int k = 0; k < RAD; k++) wa[RAD + k] = step::lds(sb + 16 + (uint32_t)k * SL);
 
-    const int zs0 = G.nbl, zs1 = G.nbl + G.nz;
+    // Plane r of the segment lies in slot r mod 8.  Groups of four planes start at slot 0 or 4:
+    // slot s of the first kind is at s0 + s SL (s < 4) or s1 + s SL (s >= 4), s0 = s1 = sb in
+    // even groups, s0 = sb + 4 SL and s1 = sb - 4 SL in odd ones, so every shared-memory access
+    // has a constant offset from one of two registers.
+    uint32_t s0 = sb, s1 = sb;
+    // From here every array is addressed by the offset kz of plane rel - 4 (stage B's), one
+    // multiply-add per access: the bases absorb the distance of the plane each one touches.
+    int kz = (zs - RAD) * NXp;
+    gu += (2 * RAD + LA) * (long long)NXp;
+    gv += (2 * RAD + LA) * (long long)NXp;
+    gd += (RAD + LA) * (long long)NXp;
+    gb += (RAD + LA) * (long long)NXp;
+    if (!IMG) u1o += RAD * (long long)NXp;
     const int warp = lx >> 5, lane = lx & 31;
-    for (int zb = zs; zb < ze; zb += U) {
-#pragma unroll
-        for (int ph = 0; ph < U; ph++) {
-            const int z = zb + ph;       // stage-A plane
-            if (z >= ze) break;
-            const int rel = z - zs;
-            const int zq = z - RAD;      // stage-B plane
-            cp_async_wait<LA - 1>();
-            __syncthreads();
-            issue_u(z + RAD + LA);
-            issue_db(z + LA);
-            cp_async_commit();
+    // Plane rel = group start + PH of stage A and, if doB (uniform), plane rel - 4 of stage B.
+    // INJ: a source or receiver may lie in one of the two planes.
+    auto plane = [&](auto phc, auto injc, int rel, bool doB) {
+        constexpr int PH = decltype(phc)::value;
+        constexpr bool INJ = decltype(injc)::value;
+        auto slot = [&](auto sc) -> uint32_t {
+            constexpr int q = decltype(sc)::value & (NR - 1);
+            return (q < U ? s0 : s1) + q * SL;
+        };
+        const uint32_t qa = slot(std::integral_constant<int, PH>{});         // plane rel
+        const uint32_t qb = slot(std::integral_constant<int, PH + RAD>{});   // planes rel - 4, rel + 4
+        cp_async_wait<LA - 1>();
+        __syncthreads();
+        issue_u(rel + RAD + LA, kz, slot(std::integral_constant<int, PH + RAD + LA>{}));
+        issue_db(rel + LA, kz, slot(std::integral_constant<int, PH + LA>{}));
+        cp_async_commit();
 
-            wa[2 * RAD + ph] = (z + RAD >= 0 && z + RAD < NZ) ? step::lds(ub + (uint32_t)((rel + RAD) & (NU - 1)) * USZ)
-                                                               : zero4;
-            const bool actA = z >= 0 && z < NZ;
-            const bool actB = zq >= z0 && zq < z1;
+        bool injA = false, injB = false;
+        if (INJ) {
             int ea0 = 0, ea1 = 0, eb0 = 0, eb1 = 0;
-            if (actA && rel >= klo && rel <= khi) {
+            const int z = zs + rel;
+            if (rel >= klo && rel <= khi && z >= 0 && z < NZ) {
                 ea0 = off[key0 + rel];
                 ea1 = off[key0 + rel + 1];
             }
-            if (actB && rel - RAD >= klo && rel - RAD <= khi) {
+            if (doB && rel - RAD >= klo && rel - RAD <= khi) {
                 eb0 = off[key0 + rel - RAD];
                 eb1 = off[key0 + rel - RAD + 1];
             }
-            const bool injA = ea1 > ea0, injB = eb1 > eb0;
+            injA = ea1 > ea0;
+            injB = eb1 > eb0;
             if (injA || injB) {
                 // each warp sums the entries of its own 128 columns (no block barrier: a
                 // lane only reads the float4 of its own columns after the warp's sync)
@@ -242,79 +256,93 @@ __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel
                 }
                 __syncwarp();
             }
+        }
 
-            // ---- stage A: step 1 at plane z on the whole tile
-            P4 u1 = zero4;
-            float sdv[4];
-            if (actA) {
-                const uint32_t az = ub + (uint32_t)(rel & (NU - 1)) * USZ;
-                const uint32_t adb = db + (uint32_t)(rel & (NDB - 1)) * DSZ;
-                const P4 wl = step::lds(az - 16), wr = step::lds(az + 16);
-                const P4 din = step::lds(adb), bb = step::lds(adb + TX * 4);
-                P4 dn, un;
-                step::step4<false, WD>(&wa[ph], nullptr, nullptr, wl, wr, din, bb, &sq[0][4 * lx], injA,
-                                   col_int && z >= zs0 && z < zs1, sdx, z, G, dn, un, sdv);
-                if (has_pad) step::zero_pad(xc, G.NX, dn, un);
-                if (a_ok) {
-                    u1 = un;
-                    step::sts(adb, dn);   // d^{n+1} replaces d^n: stage B reads it 4 planes later
-                    if (core && z >= z0 && z < z1) {
-                        const int oz = z * NXp;
-                        if (d1o) *(P4 *)(d1o + oz) = dn;
-                        if (u1o) *(P4 *)(u1o + oz) = un;
-                    }
-                }
-            }
-            step::sts(vb + (uint32_t)(rel & (NV - 1)) * VSZ, u1);
-            wb[2 * RAD + ph] = u1;
+        if (IMG && st_ok && rel >= 2 * RAD - 2 && rel + 2 < nrel) {
+            // stage B's history rows and image two planes ahead: into L2 (there are no registers
+            // or shared memory left to bring them closer)
+            const long long p = sh * A.h_ss + kz + own + 2 * (long long)NXp;
+            prefetch_l2(A.h2 + p);
+            prefetch_l2(A.h1 + p);
+            prefetch_l2(A.h0 + p);
+            prefetch_l2(A.img + sh * A.img_ss + kz + own + 2 * (long long)NXp);
+        }
+        const P4 bl = step::lds(qb + OV - 16), br = step::lds(qb + OV + 16);   // x neighbours of stage B
 
-            // ---- stage B: step 2 at plane z - 4 on the core
-            if (actB && b_ok) {
-                const int relq = rel - RAD;
-                const uint32_t av = vb + (uint32_t)(relq & (NV - 1)) * VSZ;
-                const uint32_t adb = db + (uint32_t)(relq & (NDB - 1)) * DSZ;
-                const P4 wl = step::lds(av - 16), wr = step::lds(av + 16);
-                const P4 din = step::lds(adb), bb = step::lds(adb + TX * 4);
-                P4 dn, un;
-                step::step4<false, WD>(&wb[ph], nullptr, nullptr, wl, wr, din, bb, &sq[1][4 * lx], injB,
-                                   col_int && zq >= zs0 && zq < zs1, sdx, zq, G, dn, un, sdv);
-                if (has_pad) step::zero_pad(xc, G.NX, dn, un);
-                const int oz = zq * NXp;
-                *(P4 *)(uo + oz) = un;
-                *(P4 *)(dout + oz) = dn;
+        // ---- stage A: step 1 at plane rel on the whole tile
+        wa[2 * RAD + PH] = step::lds(qb + 16);
+        const P4 al = step::lds(qa), ar = step::lds(qa + 32);
+        const P4 adin = step::lds(qa + OD), ab = step::lds(qa + OB);
+        P4 u1, d1;
+        float sdv[4];
+        step::step4<false, WD>(&wa[PH], nullptr, nullptr, al, ar, adin, ab, &sq[0][4 * lx], injA,
+                               warp_int && rel >= ri0 && rel < ri1, sdx, zs + rel, G, K, d1, u1, sdv);
+        step::sts(qa + OD, d1);   // d^{n+1} replaces d^n: stage B reads it 4 planes later
+        step::sts(qa + OV, u1);
+        wb[2 * RAD + PH] = u1;
+        if (!IMG && st_ok && rel >= RAD && rel < nrel - RAD) *(P4 *)(u1o + kz) = u1;
+
+        // ---- stage B: step 2 at plane rel - 4 on the core
+        if (doB) {
+            const P4 bdin = step::lds(qb + OD), bb = step::lds(qb + OB);
+            const P4 v1 = wb[PH + RAD];
+            P4 un, dn;
+            step::step4<false, WD>(&wb[PH], nullptr, nullptr, bl, br, bdin, bb, &sq[1][4 * lx], injB,
+                                   warp_int && rel - RAD >= ri0 && rel - RAD < ri1, sdx, zs + rel - RAD, G, K, dn, un,
+                                   sdv);
+            if (st_ok) {
+                *(P4 *)(uo + kz) = un;
+                *(P4 *)(dout + kz) = dn;
                 if (IMG) {
-                    // exact imaging of both steps at plane zq, one image read and write per
-                    // launch: first u_tt of the first step (increments h2, h1) times its
+                    // exact imaging of both steps at plane rel - 4, one image read and write
+                    // per launch: first u_tt of the first step (increments h2, h1) times its
                     // output (the window's centre), then that of the second (h1, h0) times un,
                     // each written as the one-step kernel writes its update, so a pair adds
                     // bit for bit what two single steps add
-                    float v1[4], v2[4];
-                    step::upk(wb[ph + RAD].a, v1[0], v1[1]);
-                    step::upk(wb[ph + RAD].b, v1[2], v1[3]);
+                    float v[4], v2[4];
+                    step::upk(v1.a, v[0], v[1]);
+                    step::upk(v1.b, v[2], v[3]);
                     step::upk(un.a, v2[0], v2[1]);
                     step::upk(un.b, v2[2], v2[3]);
-                    const long long p = sh * A.h_ss + oz + own;
+                    float4 *gi = (float4 *)(A.img + sh * A.img_ss + kz + own);
+                    float4 gv4 = *gi;
+                    const long long p = sh * A.h_ss + kz + own;
                     const float4 h2 = *(const float4 *)(A.h2 + p), h1 = *(const float4 *)(A.h1 + p);
                     const float4 h0 = *(const float4 *)(A.h0 + p);
-                    float4 *gi = (float4 *)(A.img + sh * A.img_ss + oz + own);
-                    float4 gv = *gi;
-                    gv.x += A.img_scale * ((1.f + sdv[0]) * h2.x - (1.f - sdv[0]) * h1.x) * v1[0];
-                    gv.y += A.img_scale * ((1.f + sdv[1]) * h2.y - (1.f - sdv[1]) * h1.y) * v1[1];
-                    gv.z += A.img_scale * ((1.f + sdv[2]) * h2.z - (1.f - sdv[2]) * h1.z) * v1[2];
-                    gv.w += A.img_scale * ((1.f + sdv[3]) * h2.w - (1.f - sdv[3]) * h1.w) * v1[3];
-                    gv.x += A.img_scale * ((1.f + sdv[0]) * h1.x - (1.f - sdv[0]) * h0.x) * v2[0];
-                    gv.y += A.img_scale * ((1.f + sdv[1]) * h1.y - (1.f - sdv[1]) * h0.y) * v2[1];
-                    gv.z += A.img_scale * ((1.f + sdv[2]) * h1.z - (1.f - sdv[2]) * h0.z) * v2[2];
-                    gv.w += A.img_scale * ((1.f + sdv[3]) * h1.w - (1.f - sdv[3]) * h0.w) * v2[3];
-                    *gi = gv;
+                    gv4.x += A.img_scale * ((1.f + sdv[0]) * h2.x - (1.f - sdv[0]) * h1.x) * v[0];
+                    gv4.y += A.img_scale * ((1.f + sdv[1]) * h2.y - (1.f - sdv[1]) * h1.y) * v[1];
+                    gv4.z += A.img_scale * ((1.f + sdv[2]) * h2.z - (1.f - sdv[2]) * h1.z) * v[2];
+                    gv4.w += A.img_scale * ((1.f + sdv[3]) * h2.w - (1.f - sdv[3]) * h1.w) * v[3];
+                    gv4.x += A.img_scale * ((1.f + sdv[0]) * h1.x - (1.f - sdv[0]) * h0.x) * v2[0];
+                    gv4.y += A.img_scale * ((1.f + sdv[1]) * h1.y - (1.f - sdv[1]) * h0.y) * v2[1];
+                    gv4.z += A.img_scale * ((1.f + sdv[2]) * h1.z - (1.f - sdv[2]) * h0.z) * v2[2];
+                    gv4.w += A.img_scale * ((1.f + sdv[3]) * h1.w - (1.f - sdv[3]) * h0.w) * v2[3];
+                    *gi = gv4;
                 }
             }
         }
+        kz += NXp;
+    };
+    auto group = [&](auto injc, int r0) {
+        const bool doB = r0 >= NR;   // stage B starts four planes after stage A's first core plane
+        plane(std::integral_constant<int, 0>{}, injc, r0, doB);
+        if (r0 + 1 < nrel) plane(std::integral_constant<int, 1>{}, injc, r0 + 1, doB);
+        if (r0 + 2 < nrel) plane(std::integral_constant<int, 2>{}, injc, r0 + 2, doB);
+        if (r0 + 3 < nrel) plane(std::integral_constant<int, 3>{}, injc, r0 + 3, doB);
+    };
+    uint32_t flip = U * SL;
+    for (int r0 = 0; r0 < nrel; r0 += U) {
+        // groups without injection entries (all but a few) run without the lookups
+        if (klo < r0 + U && khi >= r0 - RAD) group(std::true_type{}, r0);
+        else group(std::false_type{}, r0);
 #pragma unroll
         for (int k = 0; k < 2 * RAD; k++) {
             wa[k] = wa[k + U];
             wb[k] = wb[k + U];
         }
+        s0 += flip;
+        s1 -= flip;
+        flip = 0u - flip;
     }
     cp_async_wait<0>();
 }
@@ -324,7 +352,7 @@ static void launch2_variant(const GridDev &G, const StencilArgs &A, dim3 grid, c
 {
     using S = Stencil2Shape<TXT>;
     cudaFuncSetAttribute(stencil2_kernel<TXT, WD, IMG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    stencil2_kernel<TXT, WD, IMG><<<grid, S::NT, S::SMEM, s>>>(G, A);
+    pdl_launch(stencil2_kernel<TXT, WD, IMG>, grid, S::NT, S::SMEM, s, G, A);
 }
 
 template <int TXT>

@@ -103,58 +103,97 @@ __device__ __forceinline__ float rcp_approx(float x)
 
 __device__ __forceinline__ const f2 &half(const P4 &v, int p) { return p == 0 ? v.a : v.b; }
 
-// Columns i and i+1 of the 12 x-neighbour values wl | centre | wr (i in 0..10).
-__device__ __forceinline__ f2 xpair(const P4 &wl, const P4 &cc, const P4 &wr, int i)
+// Sums of the x neighbours +k and -k of the thread's four columns, pair by pair, from the 12
+// values wl | centre | wr.  Even offsets are aligned pairs (one packed add); odd offsets would
+// need both operands re-paired with register moves first, so they are two scalar adds instead:
+// the same IEEE additions.
+__device__ __forceinline__ f2 xsum(const P4 &wl, const P4 &cc, const P4 &wr, int p, int k)
 {
-    const P4 &q = i < 4 ? wl : i < 8 ? cc : wr;
-    if ((i & 1) == 0) return half(q, (i & 3) >> 1);
-    float w[12];
-    upk(wl.a, w[0], w[1]);
-    upk(wl.b, w[2], w[3]);
-    upk(cc.a, w[4], w[5]);
-    upk(cc.b, w[6], w[7]);
-    upk(wr.a, w[8], w[9]);
-    upk(wr.b, w[10], w[11]);
-    return pk(w[i], w[i + 1]);
+    const int ip = 4 + 2 * p + k, im = 4 + 2 * p - k;   // first column of either operand
+    auto quad = [&](int i) -> const P4 & { return i < 4 ? wl : i < 8 ? cc : wr; };
+    if ((k & 1) == 0) return add2(half(quad(ip), (ip & 3) >> 1), half(quad(im), (im & 3) >> 1));
+    auto col = [&](int i) {
+        float lo, hi;
+        upk(half(quad(i), (i & 3) >> 1), lo, hi);
+        return (i & 1) ? hi : lo;
+    };
+    return pk(__fadd_rn(col(ip), col(im)), __fadd_rn(col(ip + 1), col(im + 1)));
 }
 
-// One step at the four columns of the thread.  wz: own column z window with the centre at
-// wz[RAD]; wy_p / wy_m: y neighbours +k / -k (3-D only, Y = true); wl / wr: x neighbours
-// (columns -4..-1 and +4..+7); sqv: injected terms of the four columns (read if inj);
-// sdx: absorbing-layer term of the columns along x (and y); z: plane index.  Returns the
-// new increment and field; sdv receives the absorbing term of each column (0 inside).
-template <bool Y, bool WD = false>
-__device__ __forceinline__ void step4(const P4 *wz, const P4 *wy_p, const P4 *wy_m, const P4 &wl,
-                                      const P4 &wr, const P4 &din, const P4 &bb, const float *sqv,
-                                      bool inj, bool interior, const float sdx[4], int z,
-                                      const GridDev &G, P4 &dn, P4 &un, float sdv[4])
+// The step's constants as packed pairs (both halves equal): hx^2/hz^2, hx^2/hy^2, -2 (1 + rz +
+// ry), 1/hx^2 and the weights of offsets 1..4.  A packed instruction takes a constant only from
+// a register pair; built from immediates or kernel parameters the compiler re-creates the pair
+// with two moves at every use, so a kernel reads them once from shared memory (values the
+// compiler cannot re-create) and they stay in registers.
+struct Coef {
+    f2 rz, ry, nk, ih, c[4];
+};
+__device__ __forceinline__ void coef_store(f2 (*sm)[8], const GridDev &G)   // one thread, before a barrier
 {
-    const P4 &cc = wz[RAD];
-    const f2 rz = dup(G.lrz), ry = dup(G.lry), nkc0 = dup(-G.lapK), ihx2 = dup(G.ihx2);
-    f2 lap[2], wn[2];
+    const float v[8] = {G.lrz, G.lry, -G.lapK, G.ihx2, WP_C1, WP_C2, WP_C3, WP_C4};
+#pragma unroll
+    for (int i = 0; i < 8; i++) (*sm)[i] = dup(v[i]);
+}
+__device__ __forceinline__ Coef coef_load(f2 (*sm)[8])
+{
+    f2 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v[i]) : "r"((uint32_t)__cvta_generic_to_shared(&(*sm)[i])));
+    return Coef{v[0], v[1], v[2], v[3], {v[4], v[5], v[6], v[7]}};
+}
+
+// hx^2 times the Laplacian of one pair of columns: zs[k - 1], ys[k - 1] are the sums of the z and y neighbours
+// +k and -k (ys only if Y).
+template <bool Y>
+__device__ __forceinline__ f2 lap_pair(const P4 &wl, const P4 &cc, const P4 &wr, int p, const f2 zs[RAD],
+                                       const f2 ys[RAD], const Coef &K)
+{
+    const f2 c = half(cc, p);
+    f2 acc = 0ull;
+#pragma unroll
+    for (int k = 1; k <= RAD; k++) {
+        f2 sp = fma2(K.rz, zs[k - 1], xsum(wl, cc, wr, p, k));
+        if (Y) sp = fma2(K.ry, ys[k - 1], sp);
+        // centre removed with one rounding: sp - 2 (1 + rz + ry) u (the neighbour sum and
+        // the centre term nearly cancel on smooth fields)
+        const f2 t = fma2(K.nk, c, sp);
+        acc = k == 1 ? mul2(K.c[k - 1], t) : fma2(K.c[k - 1], t, acc);
+    }
+    return acc;
+}
+
+// Update of the four columns from acc = hx^2 L u.  cc: own columns of X; din: of Y; sqv:
+// injected terms (read if inj); sdx: absorbing-layer term of the columns along x (and y); z:
+// plane index.  `interior` may be false where the absorbing term is zero: the layer's form then
+// multiplies by 1 - 0 and by rcp(1) = 1 and gives the same bits.  Returns the new increment and
+// field; sdv receives the absorbing term of each column (0 inside).
+//
+// The assembler may contract a packed multiply that feeds a packed add into one fma (also with
+// .rn), differently in each kernel.  Wherever a product meets a sum, this routine therefore
+// either asks for the fma or multiplies the halves with scalar .rn instructions, which are
+// never contracted, so that every kernel gives the same bits.
+template <bool WD>
+__device__ __forceinline__ void update4(const P4 &cc, const f2 acc[2], const P4 &din, const P4 &bb, const float *sqv,
+                                        bool inj, bool interior, const float sdx[4], int z, const GridDev &G,
+                                        const Coef &K, P4 &dn, P4 &un, float sdv[4])
+{
+    f2 wn[2], lap[2];
 #pragma unroll
     for (int p = 0; p < 2; p++) {
-        const int j = 2 * p;
-        const f2 c = half(cc, p);
-        f2 acc = 0ull;
-#pragma unroll
-        for (int k = 1; k <= RAD; k++) {
-            f2 sp = add2(xpair(wl, cc, wr, 4 + j + k), xpair(wl, cc, wr, 4 + j - k));
-            sp = fma2(rz, add2(half(wz[RAD + k], p), half(wz[RAD - k], p)), sp);
-            if (Y) sp = fma2(ry, add2(half(wy_p[k - 1], p), half(wy_m[k - 1], p)), sp);
-            const f2 ck = dup(k == 1 ? WP_C1 : k == 2 ? WP_C2 : k == 3 ? WP_C3 : WP_C4);
-            // centre removed with one rounding: sp - 2 (1 + rz + ry) u (the neighbour sum and
-            // the centre term nearly cancel on smooth fields)
-            const f2 t = fma2(nkc0, c, sp);
-            acc = k == 1 ? mul2(ck, t) : fma2(ck, t, acc);
-        }
-        lap[p] = mul2(ihx2, acc);
         if (WD) {
             // w^n = w^{n-1} + L d^n; the source enters b (w^n + q) below
-            wn[p] = add2(half(din, p), lap[p]);
-            lap[p] = wn[p];
+            lap[p] = wn[p] = fma2(K.ih, acc[p], half(din, p));
+            if (inj) lap[p] = add2(lap[p], pk(sqv[2 * p], sqv[2 * p + 1]));
+        } else {
+            lap[p] = mul2(K.ih, acc[p]);
+            if (inj) {
+                float a0, a1, k0, k1;
+                upk(acc[p], a0, a1);
+                upk(K.ih, k0, k1);
+                lap[p] = add2(pk(__fmul_rn(k0, a0), __fmul_rn(k1, a1)), pk(sqv[2 * p], sqv[2 * p + 1]));
+            }
         }
-        if (inj) lap[p] = add2(lap[p], pk(sqv[j], sqv[j + 1]));
     }
     // the increment the update starts from: d^n (the own column of X in the (w, d) form)
     const P4 &dprev = WD ? cc : din;
@@ -173,7 +212,9 @@ __device__ __forceinline__ void step4(const P4 *wz, const P4 *wy_p, const P4 *wy
             const f2 t = fma2(half(bb, p), lap[p], mul2(sub2(one, sd), half(dprev, p)));
             float o0, o1;
             upk(add2(one, sd), o0, o1);
-            d[p] = mul2(t, pk(rcp_approx(o0), rcp_approx(o1)));
+            float t0, t1;
+            upk(t, t0, t1);
+            d[p] = pk(__fmul_rn(t0, rcp_approx(o0)), __fmul_rn(t1, rcp_approx(o1)));
             upk(sd, sdv[2 * p], sdv[2 * p + 1]);
         }
     }
@@ -188,6 +229,29 @@ __device__ __forceinline__ void step4(const P4 *wz, const P4 *wy_p, const P4 *wy
         un.a = add2(cc.a, d[0]);
         un.b = add2(cc.b, d[1]);
     }
+}
+
+// One step at the four columns of the thread.  wz: own column z window with the centre at
+// wz[RAD]; wy_p / wy_m: y neighbours +k / -k (3-D only, Y = true); wl / wr: x neighbours
+// (columns -4..-1 and +4..+7).
+template <bool Y, bool WD = false>
+__device__ __forceinline__ void step4(const P4 *wz, const P4 *wy_p, const P4 *wy_m, const P4 &wl,
+                                      const P4 &wr, const P4 &din, const P4 &bb, const float *sqv,
+                                      bool inj, bool interior, const float sdx[4], int z,
+                                      const GridDev &G, const Coef &K, P4 &dn, P4 &un, float sdv[4])
+{
+    f2 acc[2];
+#pragma unroll
+    for (int p = 0; p < 2; p++) {
+        f2 zs[RAD], ys[RAD];
+#pragma unroll
+        for (int k = 1; k <= RAD; k++) {
+            zs[k - 1] = add2(half(wz[RAD + k], p), half(wz[RAD - k], p));
+            ys[k - 1] = Y ? add2(half(wy_p[k - 1], p), half(wy_m[k - 1], p)) : 0ull;
+        }
+        acc[p] = lap_pair<Y>(wl, wz[RAD], wr, p, zs, ys, K);
+    }
+    update4<WD>(wz[RAD], acc, din, bb, sqv, inj, interior, sdx, z, G, K, dn, un, sdv);
 }
 
 // Zero the columns at or beyond the row length (the row padding of the internal layout).

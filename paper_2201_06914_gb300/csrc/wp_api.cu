@@ -120,6 +120,7 @@ bool build_injection(const wp_model_s *M, int nshots, int npts, const double *xy
             double w[8];
             if (!corners(M, xyz + 3 * ((size_t)s * npts + j), ix, iy, iz, w)) return false;
             for (int c = 0; c < nc; c++) {
+                if (w[c] == 0.0) continue;   // on-grid coordinate: adds nothing
                 InjEntry e;
                 const int TX = tile_x(G), TY = tile_y(G);
                 const int tile = ix[c] / TX + tiles_x(G) * (iy[c] / TY + tiles_y(G) * (iz[c] / G.tz));
@@ -167,6 +168,7 @@ bool build_injection2(const wp_model_s *M, int nshots, int npts, const double *x
             double w[8];
             if (!corners(M, xyz + 3 * ((size_t)s * npts + j), ix, iy, iz, w)) return false;
             for (int c = 0; c < nc; c++) {
+                if (w[c] == 0.0) continue;   // on-grid coordinate: adds nothing
                 for (int t = std::max(0, (ix[c] + RAD) / C - 1); t <= std::min(ntx - 1, (ix[c] + RAD) / C); t++) {
                     const int x0 = t * C - RAD;
                     if (ix[c] < x0 || ix[c] >= x0 + TX) continue;
@@ -286,12 +288,13 @@ Layout make_layout(const wp_model_s *M, const wp_geom *g, int r, int Tb, int mod
     L.t.g_idx = c.take<int>(std::max<size_t>(1, nr * nc));
     L.t.g_w = c.take<float>(std::max<size_t>(1, nr * nc));
     L.t.g_acc = c.take<double>(std::max<size_t>(1, nr * nc));
-    if (M->G.tz2 > 0) {   // an entry can fall in two tiles and two extended segments
-        const size_t ki2 = (size_t)S * (stencil2_keys(M->G) + 1);
+    if (M->G.tz2 > 0) {
+        // an entry can fall in two tiles and in every segment whose tz2 + 8 planes reach it
+        const size_t ki2 = (size_t)S * (stencil2_keys(M->G) + 1), dup = 2 * stencil2_seg_reach(M->G);
         L.t.src2_off = c.take<int>(ki2);
-        L.t.src2_ent = c.take<InjEntry>(std::max<size_t>(1, (size_t)S * g->nsrc * nc * 4));
+        L.t.src2_ent = c.take<InjEntry>(std::max<size_t>(1, (size_t)S * g->nsrc * nc * dup));
         L.t.rec2_off = c.take<int>(ki2);
-        L.t.rec2_ent = c.take<InjEntry>(std::max<size_t>(1, nr * nc * 4));
+        L.t.rec2_ent = c.take<InjEntry>(std::max<size_t>(1, nr * nc * dup));
     }
     if (M->G.tti) {
         L.t.s_idx = c.take<int>(std::max<size_t>(1, (size_t)S * g->nsrc * nc));
@@ -527,7 +530,7 @@ wp_status forward_sweep(const wp_model_s *M, const wp_geom *g, const Layout &L,
             WP_CUDA(cudaMemsetAsync(L.t.g_acc, 0, (size_t)g->nshots * g->nrec * ncorner(M->G) * sizeof(double), s));
     } else {
         A.u_in_ss = A.u_out_ss = A.gp_u_ss = 3 * N;
-        A.d_in_ss = A.d_out_ss = A.d1_ss = A.gp_d_ss = ring_ss;
+        A.d_in_ss = A.d_out_ss = A.gp_d_ss = ring_ss;
     }
     A.g_out = d_out;
     A.g_ss = (long long)nt * g->nrec;
@@ -573,15 +576,8 @@ wp_status forward_sweep(const wp_model_s *M, const wp_geom *g, const Layout &L,
         if (two) {
             A.inj_off = off2;
             A.inj = ent2;
-            if (wd) {
-                A.u1_out = slot(n + 1);
-                A.d1_out = nullptr;
-                A.u_out = slot(n + 2);
-            } else {
-                A.d1_out = slot(n + 1);
-                A.u1_out = nullptr;
-                A.d_out = slot(n + 2);
-            }
+            A.u1_out = slot(n + 1);
+            A.u_out = slot(n + 2);
             A.step2 = n + 1;
             WP_CUDA(launch_stencil2(M->G, A, s));
             if ((st = on_step(n)) != WP_OK || (st = on_step(n + 1)) != WP_OK) return st;
@@ -695,11 +691,14 @@ int choose_tz(const GridDev &G, int nshots)
     return (G.NZ + nseg - 1) / nseg;   // equal segments
 }
 
-// Planes per two-step segment (2-D isotropic grids; 0 turns two-step launches off).  A
-// segment recomputes 8 planes of its first step (4 beyond either end), so segments are
-// kept at >= 32 planes; otherwise they are sized for about four waves of resident blocks
-// (on the 64-shot 1601 x 401 model: 8 segments of 61 planes, measured fastest among
-// 25..121 planes).
+// Planes per two-step segment (2-D isotropic grids; 0 turns two-step launches off).  A launch
+// takes about (tz + 8) plane times (a segment recomputes 8 planes of its first step), and a
+// plane time grows with the load f = blocks / resident blocks.  Measured on 201 x 201 to
+// 1601 x 401 grids with 1 to 64 shots: 0.35 + 0.66 f us (throughput, plus half a plane time of
+// unevenness at the end), but 0.36 + 0.5 f us while all blocks are resident and the fields stay
+// in the L2 cache (a lone block's instruction latency, then shared issue slots).  The segment
+// length minimises the product: 3 planes for one shot of 201 x 201 (14 us a launch instead of
+// 27 at 32 planes), 8 for one of 1601 x 401 (17 instead of 25), 32 for 8 shots of it, 61 for 64.
 int choose_tz2(const GridDev &G, int nshots)
 {
     if (G.ndim != 2 || G.tti) return 0;
@@ -709,13 +708,21 @@ int choose_tz2(const GridDev &G, int nshots)
         const int v = atoi(e);
         if (v >= 1) return std::min(v, G.NZ);
     }
-    const long long cap = (long long)device_sm_count() * stencil2_blocks_per_sm(G);
-    const long long cols = (long long)tiles2_x(G) * nshots;
-    const long long segs = std::max<long long>(1, (4 * cap + cols / 2) / cols);
-    int tz = (int)((G.NZ + segs - 1) / segs);
-    tz = std::max(tz, std::min(32, G.NZ));
-    const int nseg = (G.NZ + tz - 1) / tz;
-    return (G.NZ + nseg - 1) / nseg;   // equal segments
+    const double cap = (double)device_sm_count() * stencil2_blocks_per_sm(G);
+    const double cols = (double)tiles2_x(G) * nshots;
+    const bool in_l2 = 16.0 * (double)G.Np * nshots < 129e6;   // the launch's input and output fields
+    int best = G.NZ;
+    double cost = 1e300;
+    for (int nseg = 1; nseg <= G.NZ; nseg++) {
+        const int tz = (G.NZ + nseg - 1) / nseg;
+        const double f = cols * ((G.NZ + tz - 1) / tz) / cap;
+        const double c = (tz + 2 * RAD) * (in_l2 && f <= 1 ? 0.36 + 0.5 * f : 0.35 + 0.66 * f);
+        if (c < cost) {
+            cost = c;
+            best = tz;
+        }
+    }
+    return best;
 }
 
 // The model as one call sees it: the march lengths depend on the batch size.
@@ -999,7 +1006,6 @@ wp_status wp_adjoint_image(wp_model_t *Min, const wp_geom *g, const float *resid
             A.inj_off = off2;
             A.inj = ent2;
             A.u1_out = L.ring + (size_t)(j % Tb) * RS;
-            A.d1_out = nullptr;
             A.u_out = L.ring + (size_t)((j - 1) % Tb) * RS;
             A.d_out = mu + (size_t)(dc ^ 1) * NP;
             A.step2 = j - 1;
@@ -1102,8 +1108,6 @@ wp_status wp_exact_gradient(wp_model_t *Min, const wp_geom *g, const float *wave
                 A.inj_off = roff2;
                 A.inj = rent2;
                 A.d_out = L.v + (size_t)(2 + (cd ^ 1)) * N;
-                A.u1_out = nullptr;
-                A.d1_out = nullptr;
                 A.step2 = j - 1;
                 A.h2 = hp(j + 1);
                 A.h1 = hp(j);
@@ -1138,7 +1142,7 @@ wp_status wp_exact_gradient(wp_model_t *Min, const wp_geom *g, const float *wave
             F.d_in_ss = F.d_out_ss = 3 * N;
         } else {
             F.u_in_ss = F.u_out_ss = 3 * N;
-            F.d_in_ss = F.d_out_ss = F.d1_ss = (long long)hslots * N;
+            F.d_in_ss = F.d_out_ss = (long long)hslots * N;
         }
         const int *off1 = F.inj_off;
         const InjEntry *ent1 = F.inj;
@@ -1172,14 +1176,8 @@ wp_status wp_exact_gradient(wp_model_t *Min, const wp_geom *g, const float *wave
                 if (two_ok && n + 1 < n1) {
                     F.inj_off = off2;
                     F.inj = ent2;
-                    if (wd) {
-                        F.u1_out = h_n1;
-                        F.d1_out = nullptr;
-                        F.u_out = h_n2;
-                    } else {
-                        F.d1_out = h_n1;
-                        F.d_out = h_n2;
-                    }
+                    F.u1_out = h_n1;
+                    F.u_out = h_n2;
                     F.step2 = n + 1;
                     WP_CUDA(launch_stencil2(M->G, F, s));
                     n += 2;

@@ -100,9 +100,8 @@ struct StencilArgs {
     const float *h2; const float *h1; const float *h0; long long h_ss; float img_scale;
     int nshots;
     int *err;          // device error flag (a bounded wait gave up)
-    // two-step launches (stencil2.cu): step-1 fields (NULL: kept on chip), trace row of step 2
+    // two-step launches (stencil2.cu): step-1 field X (unused with imaging), trace row of step 2
     float *u1_out; long long u1_ss;
-    float *d1_out; long long d1_ss;
     int step2;
     // pending recording row of a preceding two-step launch:
     //   out[shot*g_ss + gp_row*nrec + rec] = sum_c w[c] * (gp_u[idx[c]] + gp_d[idx[c]])
@@ -247,6 +246,8 @@ inline long long stencil_keys(const GridDev &G) { return (long long)stencil_tile
 inline int core2_x(const GridDev &G) { return G.tx - 2 * RAD; }
 inline int tiles2_x(const GridDev &G) { return (G.NXp + core2_x(G) - 1) / core2_x(G); }
 inline int tiles2_z(const GridDev &G) { return (G.NZ + G.tz2 - 1) / G.tz2; }
+// extended segments (one every tz2 planes, tz2 + 8 long) that can hold one plane
+inline int stencil2_seg_reach(const GridDev &G) { return 1 + (2 * RAD + G.tz2 - 1) / G.tz2; }
 inline int stencil2_tiles(const GridDev &G) { return tiles2_x(G) * tiles2_z(G); }
 inline long long stencil2_keys(const GridDev &G) { return (long long)stencil2_tiles(G) * (G.tz2 + 2 * RAD); }
 
@@ -370,6 +371,30 @@ int prof_read(int cls, double *total_ms, long long *count);
 void set_last_error(const char *msg);
 long long launches();
 size_t probe_gemm_smem(int r_pad);
+
+// ---------------------------------------------------------------------------------------
+// Programmatic dependent launch: a step kernel launched with pdl_launch may start while its
+// predecessor drains; it sets up its indices, lets its own successor start (pdl_trigger) and
+// waits for the predecessor's completion and memory (pdl_wait) before it touches global memory.
+// ---------------------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... KArgs, class... Args>
+inline cudaError_t pdl_launch(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, const Args &...args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
 
 // ---------------------------------------------------------------------------------------
 // PTX helpers for tcgen05 / mbarrier (sm_100a family).

@@ -1,0 +1,29 @@
+"""Two-step launches at the segment lengths where their index arithmetic has edges: segments of
+one plane and of fewer than the unrolled group's four (every entry of the injection tables then
+lies in up to nine extended segments), lengths around multiples of four and eight, one segment
+for the whole grid, grids whose last float4 of a row is padding or not, receivers on grid points
+(one non-zero corner) and between them.  A pair performs the operations of two single steps, so
+every output is bitwise that of single-step launches; the environment knobs change launch shapes
+only."""
+import numpy as np
+import pytest
+
+from paper_2201_06914_gb300.inputs import rademacher_shots
+from tests.cases import layered_case
+from tests.test_gpu_stencil2 import _run
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nx,nz,off_grid", [(108, 33, False), (237, 40, True), (512, 25, True)])
+@pytest.mark.parametrize("tz", [1, 2, 3, 4, 7, 8, 9, 16, 1000])
+def test_pairs_match_single_steps(nx, nz, off_grid, tz):
+    case = layered_case(ndim=2, nx=nx, nz=nz, nbl=8, nt=37, nshots=2, off_grid=off_grid, zi=0.3, background="const")
+    rng = np.random.default_rng(tz)
+    case.d_obs = rng.standard_normal((2, case.nt, case.rec.shape[1]))
+    Q = rademacher_shots(3, 2, case.nt, 5)
+    one = _run(case, Q, {"WP_STENCIL2": "0"}, Tb=16, ncheck=11)
+    two = _run(case, Q, {"WP_STENCIL2": "1", "WP_STENCIL2_TZ": str(tz)}, Tb=16, ncheck=11)
+    for k in one:
+        assert np.isfinite(two[k]).all(), k
+        np.testing.assert_array_equal(two[k], one[k], err_msg=k)
