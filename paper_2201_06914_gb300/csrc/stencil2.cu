@@ -55,7 +55,6 @@ namespace wp {
 using step::P4;
 using step::f2;
 
-__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 template <int TXT>
 struct Stencil2Shape {

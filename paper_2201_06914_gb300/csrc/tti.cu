@@ -13,6 +13,14 @@
 // increment-form leapfrog update of both fields, optionally the exact imaging condition
 // summed over both fields), then a point-list injection that adds the linear source term
 // to the updated increments and fields.  Both passes are tiled z-marching kernels.
+//
+// What bounds them: instruction latency at 12 to 16 warps a SM, then the latency of the planes
+// they load first; DRAM carries the passes' own bytes (28 and 64 B a point) and little more.
+// Measured (adjoint, padded 240 x 240 x 192): pass 1 85 us, 368 instructions per 128 points (93 us
+// and 582 with two points a thread), pass 2 158 us, 478 per 64 points (201 us, 661: constants
+// re-created at every use, IEEE divisions in a divergent branch, twelve copies a plane issued by
+// one thread).  One step of the padded 336 x 336 x 272 grid: 629 us (737 before), of one shot of
+// 401 x 401 in 2-D: 16.3 us (57).
 #include <cuda.h>
 
 #include <algorithm>
@@ -48,55 +56,92 @@ __device__ __forceinline__ Pt coords(const GridDev &G, long long p)
 // tiles with halos of 4 (zero outside the grid), the 9-plane z neighbourhood of a thread's
 // own points from registers.
 
+// 8-byte shared-memory load, and constants that stay in registers (a packed instruction takes a
+// constant only from a register pair; the compiler would re-create it with two moves per use).
+__device__ __forceinline__ step::f2 lds2(uint32_t addr)
+{
+    step::f2 v;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
+    return v;
+}
+
+// Differences or sums of the x neighbours +k and -k of pair p (points x + 2p, x + 2p + 1) from
+// the values f[x - 4 ..] held as aligned pairs q: even offsets are aligned pairs, odd ones two
+// scalar operations (no re-pairing moves).
+template <bool SUM>
+__device__ __forceinline__ step::f2 xpm(const step::f2 *q, int k, int p = 0)
+{
+    const int i = 2 + p;
+    if ((k & 1) == 0) return SUM ? step::add2(q[i + k / 2], q[i - k / 2]) : step::sub2(q[i + k / 2], q[i - k / 2]);
+    auto v = [&](int j) {
+        float lo, hi;
+        step::upk(q[j >> 1], lo, hi);
+        return (j & 1) ? hi : lo;
+    };
+    const int j = 2 * i;
+    return SUM ? step::pk(__fadd_rn(v(j + k), v(j - k)), __fadd_rn(v(j + 1 + k), v(j + 1 - k)))
+               : step::pk(__fsub_rn(v(j + k), v(j - k)), __fsub_rn(v(j + 1 + k), v(j + 1 - k)));
+}
+
 // Pass 1: t_j = Dr x_j = sum_i a_i D_i x_j for both fields; x_j are the fields (forward) or
 // the combinations e = E a + S b, f = S a + b (adjoint).
 //
-// Every thread owns two adjacent points of a row (one 8-byte pair) and computes both
-// fields with the packed f32x2 instructions.  The x_j tiles of a plane (with x and y
-// halos) and the a_x, a_y, a_z tiles of the block's own points are staged by 16-byte
-// cp.async copies into a ring of NS planes, LA planes ahead (zero-filled outside the
-// grid); the 9-plane z window of the own pair is kept in registers, its newest plane
-// loaded from global memory two iterations ahead.
-#ifndef WP_TTI1_LA
-#define WP_TTI1_LA 2
-#endif
-template <int TXP, int TY>
+// Every thread owns H pairs of adjacent points of a row (3-D: four points, 2-D: two) and
+// computes both fields with the packed f32x2 instructions.  The x_j tiles of a plane (with x
+// and y halos) and the a_x, a_y, a_z tiles of the block's own points are staged by 16-byte
+// cp.async copies into a ring of NS planes, LA planes ahead (zero-filled outside the grid); the
+// 9-plane z window of the own points is kept in registers, its newest plane loaded from global
+// memory two iterations ahead.
+template <int TXP, int TY, int H>
 struct Tti1Shape {
-    static constexpr int TXT = TXP / 2, NT = TXT * TY;
+    static constexpr int TXT = TXP / (2 * H), NT = TXT * TY;
     static constexpr int HY = TY > 1 ? RAD : 0;
     static constexpr int WX = TXP + 2 * RAD, WY = TY + 2 * HY;
-    static constexpr int LA = WP_TTI1_LA, NS = 4;    // planes in flight; ring slots z .. z+LA
+    static constexpr int LA = 2, NS = 4;             // planes in flight; ring slots z .. z+LA
     static constexpr int XT = WY * WX;               // floats of one field tile with halos
     static constexpr int AT = TY * TXP;              // floats of one own-point tile
     static constexpr int SLOT = 2 * XT + 3 * AT;     // x_0, x_1; a_x, a_y, a_z
     static constexpr int CH = SLOT / 4;              // 16-byte chunks per slot
     static constexpr int K = (CH + NT - 1) / NT;     // chunks per thread
-    static constexpr int U = 2;                      // planes per unrolled group
+    static constexpr int U = 2;                      // planes per unrolled group: half the ring
     static constexpr size_t SMEM = (size_t)NS * SLOT * sizeof(float);
-    static_assert(LA + 1 <= NS && (NS & (NS - 1)) == 0, "ring");
-    static_assert(TXP % 4 == 0, "tile width");
+    static constexpr int MINB = TY > 1 ? 3 : 8;      // 168 and 128 registers
+    static_assert(LA == U && NS == 2 * U, "ring");
+    static_assert(TXP % 4 == 0 && (H == 1 || H == 2), "tile width");
 };
 
-template <int TXP, int TY>
-__global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, 6) tti_pass1_kernel(const GridDev G, const TtiArgs T, int tz,
-                                                                        int ntx, int nty)
+// H pairs from shared memory in one load
+template <int H>
+__device__ __forceinline__ void ldsh(uint32_t addr, step::f2 *v)
 {
-    using S = Tti1Shape<TXP, TY>;
+    if (H == 1) v[0] = lds2(addr);
+    else {
+        const step::P4 q = step::lds(addr);
+        v[0] = q.a;
+        v[1] = q.b;
+    }
+}
+
+template <int TXP, int TY, int H>
+__global__ void __launch_bounds__(Tti1Shape<TXP, TY, H>::NT, Tti1Shape<TXP, TY, H>::MINB)
+    tti_pass1_kernel(const GridDev G, const TtiArgs T, int tz, int ntx, int nty)
+{
+    using S = Tti1Shape<TXP, TY, H>;
     using step::f2;
-    constexpr int TXT = S::TXT, NT = S::NT, HY = S::HY, WX = S::WX, XT = S::XT, AT = S::AT, LA = S::LA,
-                  NS = S::NS, U = S::U;
+    constexpr int TXT = S::TXT, NT = S::NT, HY = S::HY, WX = S::WX, XT = S::XT, AT = S::AT, LA = S::LA, U = S::U;
     constexpr uint32_t SLB = S::SLOT * 4;
     extern __shared__ float4 smem4[];
+    __shared__ f2 coef[4];
+    pdl_trigger();
+    pdl_wait();
     const int tid = threadIdx.x, lx = tid % TXT, ly = tid / TXT;
     const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, seg = blockIdx.x / (ntx * nty);
     const long long sh = blockIdx.y;
     const int x0 = bx * TXP, y0 = by * TY, z0 = seg * tz, z1 = min(z0 + tz, G.NZ);
-    const int NXp = G.NXp;
-    const long long PS = (long long)NXp * G.NY;
+    const int NXp = G.NXp, PS = G.NXp * G.NY;
     const bool adj = T.adjoint != 0;
     const float *__restrict__ f0 = adj ? T.ef_in + (2 * sh) * T.ef_ss : T.u_in + (2 * sh) * T.u_in_ss;
     const float *__restrict__ f1 = adj ? T.ef_in + (2 * sh + 1) * T.ef_ss : T.u_in + (2 * sh + 1) * T.u_in_ss;
-    float *t0 = T.t + (2 * sh) * T.t_ss, *t1 = T.t + (2 * sh + 1) * T.t_ss;
 
     // copy descriptors (fixed across planes): shared byte offset, source at plane 0, bytes
     uint32_t cd[S::K];
@@ -129,39 +174,65 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, 6) tti_pass1_kernel(co
         cb[i] = v ? 16 : 0;
     }
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem4);
-    auto issue = [&](int k) {
+    auto issue = [&](int k, uint32_t slot) {   // plane k < z1 into the slot at byte address `slot`
         if (k >= z1) return;
-        const uint32_t base = s0 + (uint32_t)((k - z0) & (NS - 1)) * SLB;
-        const long long ko = (long long)k * PS;
+        const int ko = k * PS;
 #pragma unroll
         for (int i = 0; i < S::K; i++)
-            if ((i + 1) * NT <= S::CH || tid + i * NT < S::CH) cp_async16(base + cd[i], cs[i] + ko, cb[i]);
+            if ((i + 1) * NT <= S::CH || tid + i * NT < S::CH) cp_async16(slot + cd[i], cs[i] + ko, cb[i]);
     };
 #pragma unroll
     for (int g = 0; g < LA; g++) {
-        issue(z0 + g);
+        issue(z0 + g, s0 + g * SLB);
         cp_async_commit();
     }
+    if (tid == 0) {
+        const float cw[4] = {D1C1, D1C2, D1C3, D1C4};
+#pragma unroll
+        for (int k = 0; k < 4; k++) coef[k] = step::dup(cw[k]);
+    }
 
-    const int x = x0 + 2 * lx, y = y0 + ly;
-    const bool row_ok = x < NXp && y < G.NY;      // the pair lies in the (padded) row
-    const long long own = row_ok ? (long long)y * NXp + x : 0;
-    auto ld2 = [&](const float *f, int zz) -> f2 {
-        return (row_ok && zz >= 0 && zz < G.NZ) ? *(const f2 *)(f + (long long)zz * PS + own) : 0ull;
+    const int x = x0 + 2 * H * lx, y = y0 + ly;
+    const bool row_ok = x < NXp && y < G.NY;      // the points lie in the (padded) row
+    const int own = row_ok ? y * NXp + x : 0;
+    const float *g0 = f0 + own, *g1 = f1 + own;
+    // own points of both fields at offset o (`in`: uniform; zero outside the grid)
+    auto ldw = [&](f2 *v0, f2 *v1, bool in, int o) {
+#pragma unroll
+        for (int p = 0; p < H; p++) v0[p] = v1[p] = 0ull;
+        if (!row_ok || !in) return;
+        if (H == 1) {
+            v0[0] = *(const f2 *)(g0 + o);
+            v1[0] = *(const f2 *)(g1 + o);
+        } else {
+            const step::P4 a = *(const step::P4 *)(g0 + o), b = *(const step::P4 *)(g1 + o);
+            v0[0] = a.a;
+            v0[H - 1] = a.b;
+            v1[0] = b.a;
+            v1[H - 1] = b.b;
+        }
     };
-    f2 w0[2 * RAD + U], w1[2 * RAD + U];   // w[ph + 4 + k]: plane zb + ph + k (group start zb)
+    f2 w0[2 * RAD + U][H], w1[2 * RAD + U][H];   // w[ph + 4 + k]: plane zb + ph + k (group start zb)
 #pragma unroll
     for (int k = 0; k < 2 * RAD; k++) {
-        w0[k] = ld2(f0, z0 - RAD + k);
-        w1[k] = ld2(f1, z0 - RAD + k);
+        const int zz = z0 - RAD + k;
+        ldw(w0[k], w1[k], zz >= 0 && zz < G.NZ, zz * PS);
     }
     // the newest window plane (z+4) and the one after it, loaded two iterations ahead
-    f2 p0 = ld2(f0, z0 + RAD), p1 = ld2(f1, z0 + RAD);
-    f2 n0 = ld2(f0, z0 + RAD + 1), n1 = ld2(f1, z0 + RAD + 1);
+    f2 p0[H], p1[H], n0[H], n1[H];
+    ldw(p0, p1, z0 + RAD < G.NZ, (z0 + RAD) * PS);
+    ldw(n0, n1, z0 + RAD + 1 < G.NZ, (z0 + RAD + 1) * PS);
+    float *t0 = T.t + (2 * sh) * T.t_ss + own, *t1 = T.t + (2 * sh + 1) * T.t_ss + own;
     const f2 ihx = step::dup(1.f / G.hx), ihy = step::dup(1.f / G.hy), ihz = step::dup(1.f / G.hz);
-    const float cw[4] = {D1C1, D1C2, D1C3, D1C4};
-    // pair value lanes: (x + k, x + 1 + k) of a field row from its aligned pairs
-    const int cx = (ly + HY) * WX + RAD + 2 * lx;          // float index of x in a field tile
+    const uint32_t ox = ((ly + HY) * WX + RAD + 2 * H * lx) * 4;    // own points in a field tile
+    const uint32_t oa = (2 * XT + ly * TXP + 2 * H * lx) * 4;       // and in an own-point tile
+    __syncthreads();
+    f2 ck[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) ck[k] = lds2((uint32_t)__cvta_generic_to_shared(&coef[k]));
+    const bool pad = x + 2 * H > G.NX;   // the points hold row padding: t = 0 there
+    uint32_t cur = s0, oth = s0 + U * SLB;   // the ring half of this group's planes, and the other
+    int kz = z0 * PS;
     for (int zb = z0; zb < z1; zb += U) {
 #pragma unroll
         for (int ph = 0; ph < U; ph++) {
@@ -169,66 +240,83 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, 6) tti_pass1_kernel(co
             if (z >= z1) break;
             cp_async_wait<LA - 1>();
             __syncthreads();
-            issue(z + LA);
+            issue(z + LA, oth + ph * SLB);
             cp_async_commit();
-            w0[2 * RAD + ph] = p0;
-            w1[2 * RAD + ph] = p1;
-            p0 = n0;
-            p1 = n1;
-            n0 = ld2(f0, z + RAD + 2);
-            n1 = ld2(f1, z + RAD + 2);
-            if (!row_ok) continue;
-            const uint32_t sb = s0 + (uint32_t)((z - z0) & (NS - 1)) * SLB;
-            f2 t[2];
+#pragma unroll
+            for (int p = 0; p < H; p++) {
+                w0[2 * RAD + ph][p] = p0[p];
+                w1[2 * RAD + ph][p] = p1[p];
+                p0[p] = n0[p];
+                p1[p] = n1[p];
+            }
+            ldw(n0, n1, z + RAD + 2 < G.NZ, kz + (RAD + 2) * PS);
+            const uint32_t sb = cur + ph * SLB;
+            f2 t[2][H];
 #pragma unroll
             for (int f = 0; f < 2; f++) {
-                const uint32_t fb = sb + (uint32_t)(f * XT + cx) * 4;
-                // x neighbours x-4 .. x+5 as five aligned pairs
-                f2 q[5];
+                const uint32_t fb = sb + ox + f * XT * 4;
+                f2 q[4 + H];   // x neighbours x-4 .. as aligned pairs
 #pragma unroll
-                for (int i = 0; i < 5; i++) q[i] = *(const f2 *)((const char *)smem4 + (fb - s0) + (i - 2) * 8);
-                float v[10];
-#pragma unroll
-                for (int i = 0; i < 5; i++) step::upk(q[i], v[2 * i], v[2 * i + 1]);   // v[j] = x - 4 + j
-                f2 dx = 0ull, dy = 0ull, dz = 0ull;
-                const f2 *wz = f ? w1 : w0;
+                for (int i = 0; i < 4 + H; i += H) ldsh<H>(fb + (i - 2) * 8, q + i);
+                f2 dx[H], dy[H], dz[H];
+                auto wz = f ? w1 : w0;
 #pragma unroll
                 for (int k = 1; k <= RAD; k++) {
-                    const f2 ck = step::dup(cw[k - 1]);
-                    const f2 pp = (k & 1) ? step::pk(v[4 + k], v[5 + k]) : q[2 + k / 2];
-                    const f2 pm = (k & 1) ? step::pk(v[4 - k], v[5 - k]) : q[2 - k / 2];
-                    dx = step::fma2(ck, step::sub2(pp, pm), dx);
+                    f2 yp[H], ym[H];
                     if (TY > 1) {
-                        const f2 yp = *(const f2 *)((const char *)smem4 + (fb - s0) + k * WX * 4);
-                        const f2 ym = *(const f2 *)((const char *)smem4 + (fb - s0) - k * WX * 4);
-                        dy = step::fma2(ck, step::sub2(yp, ym), dy);
+                        ldsh<H>(fb + k * WX * 4, yp);
+                        ldsh<H>(fb - k * WX * 4, ym);
                     }
-                    dz = step::fma2(ck, step::sub2(wz[ph + RAD + k], wz[ph + RAD - k]), dz);
+#pragma unroll
+                    for (int p = 0; p < H; p++) {
+                        auto acc = [&](f2 v, f2 &h) { h = k == 1 ? step::mul2(ck[0], v) : step::fma2(ck[k - 1], v, h); };
+                        acc(xpm<false>(q, k, p), dx[p]);
+                        acc(step::sub2(wz[ph + RAD + k][p], wz[ph + RAD - k][p]), dz[p]);
+                        if (TY > 1) acc(step::sub2(yp[p], ym[p]), dy[p]);
+                    }
                 }
-                const char *ab = (const char *)smem4 + (sb - s0) + (2 * XT + ly * TXP + 2 * lx) * 4;
-                const f2 axv = *(const f2 *)ab, ayv = *(const f2 *)(ab + AT * 4), azv = *(const f2 *)(ab + 2 * AT * 4);
-                f2 acc = step::mul2(step::mul2(axv, dx), ihx);
-                if (TY > 1) acc = step::fma2(step::mul2(ayv, dy), ihy, acc);
-                t[f] = step::fma2(step::mul2(azv, dz), ihz, acc);
+                f2 ax[H], ay[H], az[H];
+                ldsh<H>(sb + oa, ax);
+                if (TY > 1) ldsh<H>(sb + oa + AT * 4, ay);
+                ldsh<H>(sb + oa + 2 * AT * 4, az);
+#pragma unroll
+                for (int p = 0; p < H; p++) {
+                    f2 acc = step::mul2(step::mul2(ax[p], dx[p]), ihx);
+                    if (TY > 1) acc = step::fma2(step::mul2(ay[p], dy[p]), ihy, acc);
+                    t[f][p] = step::fma2(step::mul2(az[p], dz[p]), ihz, acc);
+                }
             }
-            if (x + 2 > G.NX) {   // row padding: t = 0
-                float a0, a1, b0, b1;
-                step::upk(t[0], a0, a1);
-                step::upk(t[1], b0, b1);
-                if (x >= G.NX) a0 = b0 = 0.f;
-                a1 = b1 = 0.f;
-                t[0] = step::pk(a0, a1);
-                t[1] = step::pk(b0, b1);
+            if (pad) {
+#pragma unroll
+                for (int f = 0; f < 2; f++)
+#pragma unroll
+                    for (int p = 0; p < H; p++) {
+                        float a, b;
+                        step::upk(t[f][p], a, b);
+                        t[f][p] = step::pk(x + 2 * p < G.NX ? a : 0.f, x + 2 * p + 1 < G.NX ? b : 0.f);
+                    }
             }
-            const long long p = (long long)z * PS + own;
-            *(f2 *)(t0 + p) = t[0];
-            *(f2 *)(t1 + p) = t[1];
+            if (row_ok) {
+                if (H == 1) {
+                    *(f2 *)(t0 + kz) = t[0][0];
+                    *(f2 *)(t1 + kz) = t[1][0];
+                } else {
+                    *(step::P4 *)(t0 + kz) = step::P4{t[0][0], t[0][H - 1]};
+                    *(step::P4 *)(t1 + kz) = step::P4{t[1][0], t[1][H - 1]};
+                }
+            }
+            kz += PS;
         }
 #pragma unroll
-        for (int k = 0; k < 2 * RAD; k++) {
-            w0[k] = w0[k + U];
-            w1[k] = w1[k + U];
-        }
+        for (int k = 0; k < 2 * RAD; k++)
+#pragma unroll
+            for (int p = 0; p < H; p++) {
+                w0[k][p] = w0[k + U][p];
+                w1[k][p] = w1[k + U][p];
+            }
+        const uint32_t sw = cur;
+        cur = oth;
+        oth = sw;
     }
     cp_async_wait<0>();
 }
@@ -237,53 +325,50 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, 6) tti_pass1_kernel(co
 // update of both fields (optionally the exact imaging condition summed over both fields).
 //
 // Every thread owns two adjacent points of a row and works on pairs with the packed f32x2
-// instructions.  One thread of the block stages each plane with tiled TMA copies
-// (cp.async.bulk.tensor, zero fill outside the grid) into a ring of NS planes, LA planes
-// ahead, completing on the slot's mbarrier: t_0, t_1 and x_0 with x and y halos, a_x with
-// the x halo, a_y with the y halo, and the block's own points of E, S, dt^2/m, both
-// increments and both fields.  The z neighbourhood of the own pair (a_z t_0, a_z t_1, x_0)
-// is a register window whose newest plane is loaded one iteration ahead.
-#ifndef WP_TTI2_U
-#define WP_TTI2_U 2
-#endif
-template <int TXP, int TY>
+// instructions (four would need 120 registers for the three windows).  Each plane is staged with
+// seven tiled TMA copies (cp.async.bulk.tensor, zero fill outside the grid) into a ring of NS
+// planes, LA planes ahead, completing on the slot's mbarrier: both t and x_0 with x and y halos,
+// a_x with the x halo, a_y with the y halo, and the block's own points of E, S and dt^2/m, of both
+// increments and of the fields.  The z neighbourhood of the own pair (a_z t_0, a_z t_1, x_0) is a
+// register window whose newest plane is loaded one iteration ahead (and in 3-D fetched into L2
+// three ahead: 3 % of a 3-D step; in 2-D the fields are in L2 already).
+template <int TXP, int TY, bool ADJ>
 struct Tti2Shape {
     static constexpr int TXT = TXP / 2, NT = TXT * TY;
     static constexpr int HY = TY > 1 ? RAD : 0;
     static constexpr int WX = TXP + 2 * RAD, WY = TY + 2 * HY;
     static constexpr int R32(int n) { return (n + 31) / 32 * 32; }   // 128-byte TMA destinations
-    static constexpr int BH = R32(WY * WX), XH = R32(TY * WX), YH = TY > 1 ? R32(WY * TXP) : 0;
-    static constexpr int OWN = R32(TY * TXP);
-    static constexpr int OT0 = 0, OT1 = BH, OX0 = 2 * BH, OAX = 3 * BH, OAY = OAX + XH, OOWN = OAY + YH;
-    static constexpr int NOWN = 7;                   // E, S, dt^2/m, d_0, d_1, a, b
-    static constexpr int SLOT = OOWN + NOWN * OWN;   // floats
-    static constexpr int LA = 2, NS = 3, U = WP_TTI2_U;
-    static constexpr uint32_t TX_BYTES = 4u * (3u * WY * WX + TY * WX + (TY > 1 ? WY * TXP : 0) + NOWN * TY * TXP);
+    static constexpr int BH = WY * WX, XH = TY * WX, YH = TY > 1 ? WY * TXP : 0, OWN = TY * TXP;
+    static constexpr int NU = ADJ ? 2 : 1;           // fields staged (forward: a is x_0's centre)
+    static constexpr int OT = 0, OX0 = R32(2 * BH), OAX = OX0 + R32(BH), OAY = OAX + R32(XH), OPAR = OAY + R32(YH),
+                         OD = OPAR + R32(3 * OWN), OU = OD + R32(2 * OWN), SLOT = OU + R32(NU * OWN);   // floats
+    static constexpr int LA = 2, NS = 3, U = 2;
+    static constexpr uint32_t TX_BYTES = 4u * (3u * BH + XH + YH + (3u + 2u + NU) * OWN);
     static constexpr size_t SMEM = (size_t)NS * SLOT * 4 + 128 + 64;
 };
 
 // Tensor maps of one pass-2 launch (encoded on the host per launch).
 struct Tti2Maps {
-    CUtensorMap t;      // [virtual shot][z][y][x] of t, box WX x WY
+    CUtensorMap t;      // [virtual shot][z][y][x] of t, box WX x WY of both fields
     CUtensorMap x0;     // x_0 field (a forward, e adjoint), box WX x WY
     CUtensorMap ax;     // [z][y][x], box WX x TY
     CUtensorMap ay;     // box TXP x WY
-    CUtensorMap E, S, bm;   // box TXP x TY
-    CUtensorMap d;      // increments [virtual shot][z][y][x], box TXP x TY
-    CUtensorMap u;      // fields, box TXP x TY
+    CUtensorMap par;    // [E, S, dt^2/m][z][y][x], box TXP x TY of all three
+    CUtensorMap d;      // increments [virtual shot][z][y][x], box TXP x TY of both fields
+    CUtensorMap u;      // fields, box TXP x TY of both (adjoint) or of b alone (forward)
 };
 
-__device__ __forceinline__ void tma3(void *dst, const CUtensorMap *map, int x, int y, int z, uint64_t *bar)
+__device__ __forceinline__ void tma3(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint64_t *bar)
 {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-                 "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+                 "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
                  "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
                  : "memory");
 }
-__device__ __forceinline__ void tma4(void *dst, const CUtensorMap *map, int x, int y, int z, int w, uint64_t *bar)
+__device__ __forceinline__ void tma4(uint32_t dst, const CUtensorMap *map, int x, int y, int z, int w, uint64_t *bar)
 {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-                 "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
+                 "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
                  "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
                  : "memory");
 }
@@ -297,219 +382,248 @@ __device__ __forceinline__ step::f2 damp_xy2(const GridDev &G, int x, int y)
 }
 
 template <int TXP, int TY, bool ADJ, bool IMG>
-__global__ void __launch_bounds__(Tti2Shape<TXP, TY>::NT, 4)
+__global__ void __launch_bounds__(Tti2Shape<TXP, TY, ADJ>::NT, TY > 1 ? 4 : 7)
     tti_pass2_kernel(const GridDev G, const TtiArgs T, int tz, int ntx, int nty, const __grid_constant__ Tti2Maps M)
 {
-    using S = Tti2Shape<TXP, TY>;
+    using S = Tti2Shape<TXP, TY, ADJ>;
     using step::f2;
     using step::pk;
     using step::upk;
     constexpr int TXT = S::TXT, HY = S::HY, WX = S::WX, LA = S::LA, NS = S::NS, U = S::U, OWN = S::OWN;
     extern __shared__ float4 smem4[];
+    __shared__ f2 coef[8];
+    __shared__ uint64_t full[NS];
     // 128-byte aligned by pointer arithmetic on the shared array (a shared pointer still)
-    float *ring = (float *)((char *)smem4 + ((128u - (smem_u32(smem4) & 127u)) & 127u));
-    uint64_t *full = (uint64_t *)(ring + NS * S::SLOT);
-    const int tid = threadIdx.x, lx = tid % TXT, ly = tid / TXT;
+    const uint32_t ring = (smem_u32(smem4) + 127u) & ~127u;
+    const int tid = threadIdx.x, lx = tid % TXT, ly = tid / TXT, warp = tid >> 5, lane = tid & 31;
     const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, seg = blockIdx.x / (ntx * nty);
     const int sh = blockIdx.y;
     const int x0 = bx * TXP, y0 = by * TY, z0 = seg * tz, z1 = min(z0 + tz, G.NZ);
-    const int NXp = G.NXp;
-    const long long PS = (long long)NXp * G.NY;
+    const int NXp = G.NXp, PS = G.NXp * G.NY;
 
     if (tid == 0) {
         for (int i = 0; i < NS; i++) mbar_init(&full[i], 1);
         fence_mbar_init();
+        const float c8[8] = {D1C1, D1C2, D1C3, D1C4, WP_C1, WP_C2, WP_C3, WP_C4};
+#pragma unroll
+        for (int k = 0; k < 8; k++) coef[k] = step::dup(c8[k]);
     }
+    pdl_trigger();
+    pdl_wait();
     __syncthreads();
-    // producer: all tiles of plane k into ring slot sl
-    int nis = 0;   // planes issued (thread 0); slot sl received nis / NS (+1 if sl < nis % NS)
+    // Producers: the seven copies of plane k into ring slot sl, shared between the warps' first
+    // lanes (one thread issuing all of them held up its warp, and the block at the barrier).
+    // The slot's phase completes once warp 0 has arrived and all bytes have landed.
+    constexpr int NW = S::NT / 32;
     auto issue = [&](int k, int sl) {
-        nis++;
-        float *b = ring + sl * S::SLOT;
+        if (lane != 0) return;
+        const uint32_t b = ring + (uint32_t)sl * (S::SLOT * 4);
         uint64_t *bar = &full[sl];
-        mbar_arrive_expect_tx(bar, S::TX_BYTES);
-        tma4(b + S::OT0, &M.t, x0 - RAD, y0 - HY, k, 2 * sh, bar);
-        tma4(b + S::OT1, &M.t, x0 - RAD, y0 - HY, k, 2 * sh + 1, bar);
-        tma4(b + S::OX0, &M.x0, x0 - RAD, y0 - HY, k, 2 * sh, bar);
-        tma3(b + S::OAX, &M.ax, x0 - RAD, y0, k, bar);
-        if (TY > 1) tma3(b + S::OAY, &M.ay, x0, y0 - HY, k, bar);
-        float *o = b + S::OOWN;
-        tma3(o + 0 * OWN, &M.E, x0, y0, k, bar);
-        tma3(o + 1 * OWN, &M.S, x0, y0, k, bar);
-        tma3(o + 2 * OWN, &M.bm, x0, y0, k, bar);
-        tma4(o + 3 * OWN, &M.d, x0, y0, k, 2 * sh, bar);
-        tma4(o + 4 * OWN, &M.d, x0, y0, k, 2 * sh + 1, bar);
-        tma4(o + 5 * OWN, &M.u, x0, y0, k, 2 * sh, bar);
-        tma4(o + 6 * OWN, &M.u, x0, y0, k, 2 * sh + 1, bar);
+        if (warp == 0) {
+            mbar_arrive_expect_tx(bar, S::TX_BYTES);
+            tma4(b + S::OT * 4, &M.t, x0 - RAD, y0 - HY, k, 2 * sh, bar);
+        }
+        if (warp == 1 % NW) {
+            tma4(b + S::OX0 * 4, &M.x0, x0 - RAD, y0 - HY, k, 2 * sh, bar);
+            tma3(b + S::OAX * 4, &M.ax, x0 - RAD, y0, k, bar);
+        }
+        if (warp == 2 % NW) {
+            if (TY > 1) tma3(b + S::OAY * 4, &M.ay, x0, y0 - HY, k, bar);
+            tma4(b + S::OPAR * 4, &M.par, x0, y0, k, 0, bar);
+        }
+        if (warp == 3 % NW) {
+            tma4(b + S::OD * 4, &M.d, x0, y0, k, 2 * sh, bar);
+            tma4(b + S::OU * 4, &M.u, x0, y0, k, ADJ ? 2 * sh : 2 * sh + 1, bar);
+        }
     };
-    if (tid == 0)
-        for (int g = 0; g < LA && z0 + g < z1; g++) issue(z0 + g, g);
+    for (int g = 0; g < LA && z0 + g < z1; g++) issue(z0 + g, g);
 
     const int x = x0 + 2 * lx, y = y0 + ly;
     const bool row_ok = x < NXp && y < G.NY;
     const bool own = row_ok && x < G.NX;          // first point of the pair inside the row
-    const long long own_off = row_ok ? (long long)y * NXp + x : 0;
-    const float *__restrict__ t0 = T.t + (2LL * sh) * T.t_ss;
-    const float *__restrict__ t1 = T.t + (2LL * sh + 1) * T.t_ss;
-    const float *__restrict__ xf = ADJ ? T.ef_in + (2LL * sh) * T.ef_ss : T.u_in + (2LL * sh) * T.u_in_ss;
+    const int off = row_ok ? y * NXp + x : 0;
+    const float *__restrict__ t0 = T.t + (2LL * sh) * T.t_ss + off;
+    const float *__restrict__ t1 = T.t + (2LL * sh + 1) * T.t_ss + off;
+    const float *__restrict__ xf = (ADJ ? T.ef_in + (2LL * sh) * T.ef_ss : T.u_in + (2LL * sh) * T.u_in_ss) + off;
+    const float *__restrict__ azf = T.az + off;
     auto ld2 = [&](const float *f, int zz) -> f2 {
-        return (row_ok && zz >= 0 && zz < G.NZ) ? *(const f2 *)(f + (long long)zz * PS + own_off) : 0ull;
+        return (row_ok && zz >= 0 && zz < G.NZ) ? *(const f2 *)(f + zz * PS) : 0ull;
     };
     // z windows: a_z t_0, a_z t_1, x_0 of plane zb + i - 4 at index i (group start zb)
     f2 wa[2 * RAD + U], wb[2 * RAD + U], wx[2 * RAD + U];
 #pragma unroll
     for (int k = 0; k < 2 * RAD; k++) {
         const int zz = z0 - RAD + k;
-        const f2 az = ld2(T.az, zz);
+        const f2 az = ld2(azf, zz);
         wa[k] = step::mul2(az, ld2(t0, zz));
         wb[k] = step::mul2(az, ld2(t1, zz));
         wx[k] = ld2(xf, zz);
     }
-    f2 qa = ld2(T.az, z0 + RAD), q0 = ld2(t0, z0 + RAD), q1 = ld2(t1, z0 + RAD), qx = ld2(xf, z0 + RAD);
-    float *uo0 = T.u_out + (2LL * sh) * T.u_out_ss, *uo1 = T.u_out + (2LL * sh + 1) * T.u_out_ss;
-    float *do0 = T.d_out + (2LL * sh) * T.d_out_ss, *do1 = T.d_out + (2LL * sh + 1) * T.d_out_ss;
-    float *eo = ADJ ? T.ef_out + (2LL * sh) * T.ef_ss : nullptr;
-    float *fo = ADJ ? T.ef_out + (2LL * sh + 1) * T.ef_ss : nullptr;
+    f2 qa = ld2(azf, z0 + RAD), q0 = ld2(t0, z0 + RAD), q1 = ld2(t1, z0 + RAD), qx = ld2(xf, z0 + RAD);
+    float *uo0 = T.u_out + (2LL * sh) * T.u_out_ss + off, *uo1 = T.u_out + (2LL * sh + 1) * T.u_out_ss + off;
+    float *do0 = T.d_out + (2LL * sh) * T.d_out_ss + off, *do1 = T.d_out + (2LL * sh + 1) * T.d_out_ss + off;
+    float *eo = ADJ ? T.ef_out + (2LL * sh) * T.ef_ss + off : nullptr;
+    float *fo = ADJ ? T.ef_out + (2LL * sh + 1) * T.ef_ss + off : nullptr;
     const f2 ihx = step::dup(1.f / G.hx), ihy = step::dup(1.f / G.hy), ihz = step::dup(1.f / G.hz);
     const f2 ihx2 = step::dup(G.ihx2), ihy2 = step::dup(G.ihy2), ihz2 = step::dup(G.ihz2);
-    const f2 two = step::dup(2.f), one = step::dup(1.f);
-    const float cw[4] = {D1C1, D1C2, D1C3, D1C4};
-    const float lw[4] = {WP_C1, WP_C2, WP_C3, WP_C4};
-    const int cb = (ly + HY) * WX + RAD + 2 * lx;   // own pair in a both-halo tile
-    const int cxh = ly * WX + RAD + 2 * lx;         // own pair in the a_x tile
-    const int cyh = (ly + HY) * TXP + 2 * lx;       // own pair in the a_y tile
-    const int co = ly * TXP + 2 * lx;               // own pair in an own-point tile
+    f2 cw[4], lw[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        cw[k] = lds2(smem_u32(&coef[k]));
+        lw[k] = lds2(smem_u32(&coef[4 + k]));
+    }
+    const uint32_t ob = ((ly + HY) * WX + RAD + 2 * lx) * 4;   // own pair in a both-halo tile
+    const uint32_t oxh = (ly * WX + RAD + 2 * lx) * 4;         // own pair in the a_x tile
+    const uint32_t oyh = ((ly + HY) * TXP + 2 * lx) * 4;       // own pair in the a_y tile
+    const uint32_t oo = (ly * TXP + 2 * lx) * 4;               // own pair in an own-point tile
     const f2 sdxy = damp_xy2(G, x, y);
+    // Absorbing layer, s = sigma dt / 2: the update divides by 1 + s.  With rc the correctly
+    // rounded reciprocal of c = 1 + s, q = t rc corrected once by its exact remainder, q + (t -
+    // c q) rc, is the correctly rounded quotient (Markstein 1990), and t itself where s = 0: three
+    // packed operations at every point instead of a branch around IEEE divisions.  c, rc and
+    // 1 - s change only in planes of the z layers.
+    f2 cp, ncp, rc, cm;
+    auto layer = [&](int z) {
+        const f2 sd = step::add2(sdxy, step::dup(damp_term(z, G.nz, G.nbl, G.hs0z, G.inv_nbl)));
+        float c0, c1;
+        cp = step::add2(step::dup(1.f), sd);
+        cm = step::sub2(step::dup(1.f), sd);
+        upk(cp, c0, c1);
+        ncp = pk(-c0, -c1);
+        rc = pk(__frcp_rn(c0), __frcp_rn(c1));
+    };
+    layer(z0);
+    const int zl0 = G.nbl, zl1 = G.nbl + G.nz;   // planes zl0 .. zl1 - 1 lie between the z layers
+    const bool pad = x + 2 > G.NX;               // the pair holds row padding: kept at zero
     bool failed = false;
-    int sc = 0;                                     // ring slot of plane z
+    int sc = 0;                                  // ring slot of plane z
+    uint32_t parity = 0, slot = ring;
+    int kz = z0 * PS;
     for (int zb = z0; zb < z1; zb += U) {
 #pragma unroll
         for (int ph = 0; ph < U; ph++) {
             const int z = zb + ph;
             if (z >= z1) break;
-            if (__syncthreads_or(failed)) goto done;   // slot of plane z-1 is free again
-            if (tid == 0 && z + LA < z1) issue(z + LA, sc + LA >= NS ? sc + LA - NS : sc + LA);
+            __syncthreads();   // slot of plane z-1 is free again
+            if (z + LA < z1) issue(z + LA, sc + LA >= NS ? sc + LA - NS : sc + LA);
             // own pair of plane z+4 enters the windows; plane z+5 is loaded
             wa[2 * RAD + ph] = step::mul2(qa, q0);
             wb[2 * RAD + ph] = step::mul2(qa, q1);
             wx[2 * RAD + ph] = qx;
-            qa = ld2(T.az, z + RAD + 1);
-            q0 = ld2(t0, z + RAD + 1);
-            q1 = ld2(t1, z + RAD + 1);
-            qx = ld2(xf, z + RAD + 1);
-            const uint32_t parity = (uint32_t)(((z - z0) / NS) & 1);
-            if (!mbar_wait_bounded(&full[sc], parity)) {
+            qa = q0 = q1 = qx = 0ull;
+            if (row_ok && z + RAD + 1 < G.NZ) {
+                const int k5 = kz + (RAD + 1) * PS;
+                qa = *(const f2 *)(azf + k5);
+                q0 = *(const f2 *)(t0 + k5);
+                q1 = *(const f2 *)(t1 + k5);
+                qx = *(const f2 *)(xf + k5);
+            }
+            if (TY > 1 && row_ok && z + RAD + 3 < G.NZ) {   // the window's planes two further, into L2
+                const int k7 = kz + (RAD + 3) * PS;
+                prefetch_l2(azf + k7);
+                prefetch_l2(t0 + k7);
+                prefetch_l2(t1 + k7);
+                prefetch_l2(xf + k7);
+            }
+            if (z <= zl0 || z >= zl1) layer(z);
+            // a wait that gives up sets the error flag; the march goes on without waiting
+            if (!failed && !mbar_wait_bounded(&full[sc], parity)) {
                 failed = true;
                 if (T.err) atomicExch(T.err, 1);
             }
-            if (!failed && row_ok) {
-                const float *sl = ring + sc * S::SLOT;
-                const float *o = sl + S::OOWN;
-                // x parts: five aligned pairs x-4 .. x+5 of t_0, t_1, x_0 and a_x
-                f2 p0[5], p1[5], px[5];
+            // x parts: five aligned pairs x-4 .. x+5 of t_0, t_1, x_0 and a_x
+            f2 p0[5], p1[5], px[5];
 #pragma unroll
-                for (int i = 0; i < 5; i++) {
-                    const f2 a = *(const f2 *)(sl + S::OAX + cxh + 2 * i - 4);
-                    p0[i] = step::mul2(a, *(const f2 *)(sl + S::OT0 + cb + 2 * i - 4));
-                    p1[i] = step::mul2(a, *(const f2 *)(sl + S::OT1 + cb + 2 * i - 4));
-                    px[i] = *(const f2 *)(sl + S::OX0 + cb + 2 * i - 4);
-                }
-                auto shifted = [&](const f2 *q, int k) -> f2 {   // (v[x+k], v[x+1+k]), k in -4..4
-                    if ((k & 1) == 0) return q[2 + k / 2];
-                    float lo0, hi0, lo1, hi1;
-                    const int i = (k + 3) >> 1;                 // pair holding x+k as its second lane
-                    upk(q[i + 1], lo1, hi1);
-                    upk(q[i], lo0, hi0);
-                    return pk(hi0, lo1);
-                };
-                const f2 c = px[2];
-                f2 hx0 = 0ull, hx1 = 0ull, lxx = 0ull, hy0 = 0ull, hy1 = 0ull, lyy = 0ull, hz0 = 0ull, hz1 = 0ull, lzz = 0ull;
+            for (int i = 0; i < 5; i++) {
+                const f2 a = lds2(slot + oxh + S::OAX * 4 + (i - 2) * 8);
+                p0[i] = step::mul2(a, lds2(slot + ob + S::OT * 4 + (i - 2) * 8));
+                p1[i] = step::mul2(a, lds2(slot + ob + (S::OT + S::BH) * 4 + (i - 2) * 8));
+                px[i] = lds2(slot + ob + S::OX0 * 4 + (i - 2) * 8);
+            }
+            const f2 c = px[2], c2 = step::add2(c, c);
+            f2 hx0, hx1, lxx, hy0 = 0ull, hy1 = 0ull, lyy = 0ull, hz0, hz1, lzz;
 #pragma unroll
-                for (int k = 1; k <= RAD; k++) {
-                    const f2 cf = step::dup(cw[k - 1]), lf = step::dup(lw[k - 1]);
-                    hx0 = step::fma2(cf, step::sub2(shifted(p0, k), shifted(p0, -k)), hx0);
-                    hx1 = step::fma2(cf, step::sub2(shifted(p1, k), shifted(p1, -k)), hx1);
-                    lxx = step::fma2(lf, step::sub2(step::add2(shifted(px, k), shifted(px, -k)), step::mul2(two, c)), lxx);
-                    if (TY > 1) {
-                        const f2 ap = *(const f2 *)(sl + S::OAY + cyh + k * TXP);
-                        const f2 am = *(const f2 *)(sl + S::OAY + cyh - k * TXP);
-                        const f2 y0p = step::mul2(ap, *(const f2 *)(sl + S::OT0 + cb + k * WX));
-                        const f2 y0m = step::mul2(am, *(const f2 *)(sl + S::OT0 + cb - k * WX));
-                        const f2 y1p = step::mul2(ap, *(const f2 *)(sl + S::OT1 + cb + k * WX));
-                        const f2 y1m = step::mul2(am, *(const f2 *)(sl + S::OT1 + cb - k * WX));
-                        hy0 = step::fma2(cf, step::sub2(y0p, y0m), hy0);
-                        hy1 = step::fma2(cf, step::sub2(y1p, y1m), hy1);
-                        const f2 xp = *(const f2 *)(sl + S::OX0 + cb + k * WX);
-                        const f2 xm = *(const f2 *)(sl + S::OX0 + cb - k * WX);
-                        lyy = step::fma2(lf, step::sub2(step::add2(xp, xm), step::mul2(two, c)), lyy);
-                    }
-                    hz0 = step::fma2(cf, step::sub2(wa[ph + RAD + k], wa[ph + RAD - k]), hz0);
-                    hz1 = step::fma2(cf, step::sub2(wb[ph + RAD + k], wb[ph + RAD - k]), hz1);
-                    lzz = step::fma2(lf, step::sub2(step::add2(wx[ph + RAD + k], wx[ph + RAD - k]), step::mul2(two, c)), lzz);
-                }
-                f2 H0 = step::mul2(hx0, ihx), H1 = step::mul2(hx1, ihx), lap = step::mul2(lxx, ihx2);
+            for (int k = 1; k <= RAD; k++) {
+                const f2 cf = cw[k - 1], lf = lw[k - 1];
+                auto acc = [&](f2 co, f2 v, f2 &h) { h = k == 1 ? step::mul2(co, v) : step::fma2(co, v, h); };
+                acc(cf, xpm<false>(p0, k), hx0);
+                acc(cf, xpm<false>(p1, k), hx1);
+                acc(lf, step::sub2(xpm<true>(px, k), c2), lxx);
                 if (TY > 1) {
-                    H0 = step::fma2(hy0, ihy, H0);
-                    H1 = step::fma2(hy1, ihy, H1);
-                    lap = step::fma2(lyy, ihy2, lap);
+                    const f2 ap = lds2(slot + oyh + (S::OAY + k * TXP) * 4);
+                    const f2 am = lds2(slot + oyh + (S::OAY - k * TXP) * 4);
+                    const f2 y0p = step::mul2(ap, lds2(slot + ob + (S::OT + k * WX) * 4));
+                    const f2 y0m = step::mul2(am, lds2(slot + ob + (S::OT - k * WX) * 4));
+                    const f2 y1p = step::mul2(ap, lds2(slot + ob + (S::OT + S::BH + k * WX) * 4));
+                    const f2 y1m = step::mul2(am, lds2(slot + ob + (S::OT + S::BH - k * WX) * 4));
+                    acc(cf, step::sub2(y0p, y0m), hy0);
+                    acc(cf, step::sub2(y1p, y1m), hy1);
+                    const f2 xp = lds2(slot + ob + (S::OX0 + k * WX) * 4), xm = lds2(slot + ob + (S::OX0 - k * WX) * 4);
+                    acc(lf, step::sub2(step::add2(xp, xm), c2), lyy);
                 }
-                H0 = step::fma2(hz0, ihz, H0);
-                H1 = step::fma2(hz1, ihz, H1);
-                lap = step::fma2(lzz, ihz2, lap);
-                const f2 cE = *(const f2 *)(o + 0 * OWN + co), cS = *(const f2 *)(o + 1 * OWN + co);
-                const f2 cbm = *(const f2 *)(o + 2 * OWN + co);
-                const f2 cd0 = *(const f2 *)(o + 3 * OWN + co), cd1 = *(const f2 *)(o + 4 * OWN + co);
-                const f2 ca = *(const f2 *)(o + 5 * OWN + co), cbv = *(const f2 *)(o + 6 * OWN + co);
-                f2 r0, r1;
-                if (!ADJ) {
-                    const f2 h0p = step::sub2(lap, H0);
-                    r0 = step::fma2(cE, h0p, step::mul2(cS, H1));
-                    r1 = step::fma2(cS, h0p, H1);
-                } else {
-                    r0 = step::sub2(lap, H0);
-                    r1 = H1;
-                }
-                const f2 sd = step::add2(sdxy, step::dup(damp_term(z, G.nz, G.nbl, G.hs0z, G.inv_nbl)));
-                const f2 cp = step::add2(one, sd), cm = step::sub2(one, sd);
-                f2 dn0 = step::fma2(cbm, r0, step::mul2(cm, cd0));
-                f2 dn1 = step::fma2(cbm, r1, step::mul2(cm, cd1));
-                if (sd != 0ull) {   // inside the absorbing layer: divide by 1 + s
-                    float a0, a1, b0, b1, c0, c1;
-                    upk(dn0, a0, a1);
-                    upk(dn1, b0, b1);
-                    upk(cp, c0, c1);
-                    dn0 = pk(a0 / c0, a1 / c1);
-                    dn1 = pk(b0 / c0, b1 / c1);
-                }
-                f2 un0 = step::add2(ca, dn0), un1 = step::add2(cbv, dn1);
-                f2 e2 = 0ull, f2v = 0ull;
+                acc(cf, step::sub2(wa[ph + RAD + k], wa[ph + RAD - k]), hz0);
+                acc(cf, step::sub2(wb[ph + RAD + k], wb[ph + RAD - k]), hz1);
+                acc(lf, step::sub2(step::add2(wx[ph + RAD + k], wx[ph + RAD - k]), c2), lzz);
+            }
+            f2 H0 = step::mul2(hx0, ihx), H1 = step::mul2(hx1, ihx), lap = step::mul2(lxx, ihx2);
+            if (TY > 1) {
+                H0 = step::fma2(hy0, ihy, H0);
+                H1 = step::fma2(hy1, ihy, H1);
+                lap = step::fma2(lyy, ihy2, lap);
+            }
+            H0 = step::fma2(hz0, ihz, H0);
+            H1 = step::fma2(hz1, ihz, H1);
+            lap = step::fma2(lzz, ihz2, lap);
+            const uint32_t po = slot + oo;
+            const f2 cE = lds2(po + S::OPAR * 4), cS = lds2(po + (S::OPAR + OWN) * 4);
+            const f2 cbm = lds2(po + (S::OPAR + 2 * OWN) * 4);
+            const f2 cd0 = lds2(po + S::OD * 4), cd1 = lds2(po + (S::OD + OWN) * 4);
+            const f2 ca = ADJ ? lds2(po + S::OU * 4) : c, cbv = lds2(po + (S::OU + (ADJ ? OWN : 0)) * 4);
+            f2 r0, r1;
+            if (!ADJ) {
+                const f2 h0p = step::sub2(lap, H0);
+                r0 = step::fma2(cE, h0p, step::mul2(cS, H1));
+                r1 = step::fma2(cS, h0p, H1);
+            } else {
+                r0 = step::sub2(lap, H0);
+                r1 = H1;
+            }
+            auto update = [&](f2 r, f2 dprev) {
+                const f2 t = step::fma2(cbm, r, step::mul2(cm, dprev));
+                const f2 q = step::mul2(t, rc);
+                return step::fma2(step::fma2(ncp, q, t), rc, q);
+            };
+            f2 dn0 = update(r0, cd0), dn1 = update(r1, cd1);
+            f2 un0 = step::add2(ca, dn0), un1 = step::add2(cbv, dn1);
+            f2 e2 = 0ull, f2v = 0ull;
+            if (ADJ) {
+                e2 = step::fma2(cE, un0, step::mul2(cS, un1));
+                f2v = step::fma2(cS, un0, un1);
+            }
+            if (pad) {
+                auto padz = [&](f2 &v) {
+                    float lo, hi;
+                    upk(v, lo, hi);
+                    v = pk(own ? lo : 0.f, 0.f);
+                };
+                padz(un0);
+                padz(un1);
+                padz(dn0);
+                padz(dn1);
+                padz(e2);
+                padz(f2v);
+            }
+            if (row_ok) {
+                *(f2 *)(uo0 + kz) = un0;
+                *(f2 *)(uo1 + kz) = un1;
+                *(f2 *)(do0 + kz) = dn0;
+                *(f2 *)(do1 + kz) = dn1;
                 if (ADJ) {
-                    e2 = step::fma2(cE, un0, step::mul2(cS, un1));
-                    f2v = step::fma2(cS, un0, un1);
-                }
-                if (x + 2 > G.NX) {   // row padding: kept at zero
-                    auto pad = [&](f2 &v) {
-                        float lo, hi;
-                        upk(v, lo, hi);
-                        v = pk(own ? lo : 0.f, 0.f);
-                    };
-                    pad(un0);
-                    pad(un1);
-                    pad(dn0);
-                    pad(dn1);
-                    pad(e2);
-                    pad(f2v);
-                }
-                const long long p = (long long)z * PS + own_off;
-                *(f2 *)(uo0 + p) = un0;
-                *(f2 *)(uo1 + p) = un1;
-                *(f2 *)(do0 + p) = dn0;
-                *(f2 *)(do1 + p) = dn1;
-                if (ADJ) {
-                    *(f2 *)(eo + p) = e2;
-                    *(f2 *)(fo + p) = f2v;
+                    *(f2 *)(eo + kz) = e2;
+                    *(f2 *)(fo + kz) = f2v;
                 }
                 if (IMG) {
+                    const long long p = kz + off;
                     const float *h1a = T.h1 + (2LL * sh) * T.h_ss, *h0a = T.h0 + (2LL * sh) * T.h_ss;
                     const float *h1b = T.h1 + (2LL * sh + 1) * T.h_ss, *h0b = T.h0 + (2LL * sh + 1) * T.h_ss;
                     const f2 ua = step::sub2(step::mul2(cp, *(const f2 *)(h1a + p)), step::mul2(cm, *(const f2 *)(h0a + p)));
@@ -517,7 +631,7 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY>::NT, 4)
                     f2 *gi = (f2 *)(T.img + (long long)sh * T.img_ss + p);
                     const f2 add = step::mul2(step::dup(T.img_scale), step::fma2(ua, un0, step::mul2(ub, un1)));
                     f2 g = step::add2(*gi, add);
-                    if (x + 2 > G.NX) {
+                    if (pad) {
                         float lo, hi;
                         upk(g, lo, hi);
                         g = pk(own ? lo : 0.f, 0.f);
@@ -525,7 +639,14 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY>::NT, 4)
                     *gi = g;
                 }
             }
-            sc = sc + 1 == NS ? 0 : sc + 1;
+            kz += PS;
+            sc++;
+            slot += S::SLOT * 4;
+            if (sc == NS) {
+                sc = 0;
+                slot = ring;
+                parity ^= 1;
+            }
         }
 #pragma unroll
         for (int k = 0; k < 2 * RAD; k++) {
@@ -534,11 +655,10 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY>::NT, 4)
             wx[k] = wx[k + U];
         }
     }
-done:
     // after a failed wait, let the copies in flight land before the block's memory is reused
     if (__syncthreads_or(failed) && tid == 0)
         for (int i = 0; i < NS; i++) {
-            const int cnt = nis / NS + (i < nis % NS ? 1 : 0);
+            const int n = z1 - z0, cnt = n / NS + (i < n % NS ? 1 : 0);   // planes issued into slot i
             if (cnt > 0) (void)mbar_wait_bounded(&full[i], (uint32_t)((cnt - 1) & 1));
         }
     __syncthreads();
@@ -552,6 +672,8 @@ __global__ void tti_inject_kernel(const GridDev G, const TtiArgs T, const int *i
                                   int npts, int ncorner, const float *traces, long long tr_ss,
                                   long long tr_ts, long long tr_rs, int step, float sign, int both)
 {
+    pdl_trigger();
+    pdl_wait();
     const long long sh = blockIdx.y;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= npts * ncorner) return;
@@ -614,98 +736,76 @@ cudaError_t launch_tti_params(const GridDev &G, const float *eps, const float *d
     return cudaGetLastError();
 }
 
-typedef CUresult (*tti_encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-
-static tti_encode_fn tti_encoder()
-{
-    static tti_encode_fn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (tti_encode_fn)p;
-    }
-    return fn;
-}
-
-// A tiled float map over [w][z][y][x] (rank 4, w_ss floats between w slices) or [z][y][x]
-// (rank 3) of a padded field; out-of-range elements read as zero.
+// A tiled float map over [w][z][y][x] (rank 4, w_ss floats between w slices, boxes of bw of
+// them) or [z][y][x] (rank 3) of a padded field; out-of-range elements read as zero.
 static bool tti_map(CUtensorMap *m, const float *base, const GridDev &G, int rank, long long nw, long long w_ss,
-                    uint32_t bx, uint32_t by)
+                    uint32_t bx, uint32_t by, uint32_t bw = 1)
 {
-    tti_encode_fn enc = tti_encoder();
+    encode_tiled_fn enc = encoder();
     if (!enc || ((uintptr_t)base & 15) || (w_ss & 3)) return false;
     const cuuint64_t dims[4] = {(cuuint64_t)G.NXp, (cuuint64_t)G.NY, (cuuint64_t)G.NZ, (cuuint64_t)nw};
     const cuuint64_t strides[3] = {(cuuint64_t)G.NXp * 4, (cuuint64_t)G.NXp * G.NY * 4, (cuuint64_t)w_ss * 4};
-    const cuuint32_t box[4] = {bx, by, 1, 1};
+    const cuuint32_t box[4] = {bx, by, 1, bw};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, (void *)base, dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int TX, int TY>
+// TX x TY: tile of pass 2; TX x TY1 and H1 pairs per thread: of pass 1.
+template <int TX, int TY, int TY1, int H1, bool ADJ>
 static cudaError_t tti_passes(const GridDev &G, const TtiArgs &T, cudaStream_t s)
 {
-    const int ntx = (G.NX + TX - 1) / TX, nty = (G.NY + TY - 1) / TY;
-    // z segments: about four waves of 8 resident blocks per SM, marches of >= 16 planes
-    const long long cols = (long long)ntx * nty * T.nshots;
-    const long long want = 4LL * device_sm_count() * 8;
-    int nseg = (int)std::max<long long>(1, (want + cols - 1) / cols);
-    int tz = (G.NZ + nseg - 1) / nseg;
-    tz = std::max(tz, std::min(16, G.NZ));
-    nseg = (G.NZ + tz - 1) / tz;
+    using S1 = Tti1Shape<TX, TY1, H1>;
+    const int ntx = (G.NX + TX - 1) / TX, nty = (G.NY + TY - 1) / TY, nty1 = (G.NY + TY1 - 1) / TY1;
+    // z segments: a march costs its planes and about five more for the z windows' first planes,
+    // and a plane time grows with the load (choose_segment).  One shot of 401 x 401 takes 3 planes
+    // (16.8 us a step; 30.2 at the former least of 16), of 1601 x 401 6 (24.5; 36.7), 256^3 about
+    // 30 (within 2 % of the best of 12 .. 136).
+    const int tz = choose_segment(G.NZ, (double)ntx * nty * T.nshots, (double)device_sm_count() * (TY > 1 ? 4 : 7), 5.0);
+    const int nseg = (G.NZ + tz - 1) / tz;
     dim3 grid((unsigned)((long long)ntx * nty * nseg), T.nshots);
-    using S1 = Tti1Shape<TX, TY>;
-    cudaFuncSetAttribute(tti_pass1_kernel<TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S1::SMEM);
-    tti_pass1_kernel<TX, TY><<<grid, S1::NT, S1::SMEM, s>>>(G, T, tz, ntx, nty);
+    cudaFuncSetAttribute(tti_pass1_kernel<TX, TY1, H1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S1::SMEM);
+    dim3 grid1((unsigned)((long long)ntx * nty1 * nseg), T.nshots);
+    pdl_launch(tti_pass1_kernel<TX, TY1, H1>, grid1, S1::NT, S1::SMEM, s, G, T, tz, ntx, nty1);
 
-    using S2 = Tti2Shape<TX, TY>;
+    using S2 = Tti2Shape<TX, TY, ADJ>;
     Tti2Maps M;
     memset(&M, 0, sizeof M);
     const long long nv = 2LL * T.nshots;
-    const float *xf = T.adjoint ? T.ef_in : T.u_in;
-    const long long xss = T.adjoint ? T.ef_ss : T.u_in_ss;
-    bool ok = tti_map(&M.t, T.t, G, 4, nv, T.t_ss, S2::WX, S2::WY) &&
+    const float *xf = ADJ ? T.ef_in : T.u_in;
+    const long long xss = ADJ ? T.ef_ss : T.u_in_ss;
+    const long long pss = T.Sd - T.E;   // E, S and dt^2/m lie one after the other
+    if (T.b - T.Sd != pss) return cudaErrorInvalidValue;
+    bool ok = tti_map(&M.t, T.t, G, 4, nv, T.t_ss, S2::WX, S2::WY, 2) &&
               tti_map(&M.x0, xf, G, 4, nv, xss, S2::WX, S2::WY) &&
               tti_map(&M.ax, T.ax, G, 3, 1, 0, S2::WX, TY) &&
               tti_map(&M.ay, T.ay, G, 3, 1, 0, TX, S2::WY) &&
-              tti_map(&M.E, T.E, G, 3, 1, 0, TX, TY) && tti_map(&M.S, T.Sd, G, 3, 1, 0, TX, TY) &&
-              tti_map(&M.bm, T.b, G, 3, 1, 0, TX, TY) &&
-              tti_map(&M.d, T.d_in, G, 4, nv, T.d_in_ss, TX, TY) &&
-              tti_map(&M.u, T.u_in, G, 4, nv, T.u_in_ss, TX, TY);
+              tti_map(&M.par, T.E, G, 4, 3, pss, TX, TY, 3) &&
+              tti_map(&M.d, T.d_in, G, 4, nv, T.d_in_ss, TX, TY, 2) &&
+              tti_map(&M.u, T.u_in, G, 4, nv, T.u_in_ss, TX, TY, S2::NU);
     if (!ok) return cudaErrorInvalidValue;
     auto run = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);
-        kern<<<grid, S2::NT, S2::SMEM, s>>>(G, T, tz, ntx, nty, M);
+        pdl_launch(kern, grid, S2::NT, S2::SMEM, s, G, T, tz, ntx, nty, M);
     };
-    if (T.img) {
-        if (T.adjoint) run(tti_pass2_kernel<TX, TY, true, true>);
-        else run(tti_pass2_kernel<TX, TY, false, true>);
-    } else {
-        if (T.adjoint) run(tti_pass2_kernel<TX, TY, true, false>);
-        else run(tti_pass2_kernel<TX, TY, false, false>);
-    }
+    if (ADJ && T.img) run(tti_pass2_kernel<TX, TY, true, true>);
+    else run(tti_pass2_kernel<TX, TY, ADJ, false>);
     return cudaSuccess;
 }
 
 cudaError_t launch_tti_step(const GridDev &G, const TtiArgs &T, const TtiInject &J, cudaStream_t s)
 {
     cudaEvent_t ev = prof_begin(PROF_STENCIL, s);
-    const cudaError_t e = G.ndim == 3 ? tti_passes<32, 8>(G, T, s) : tti_passes<128, 1>(G, T, s);
+    if (T.img && !T.adjoint) return cudaErrorInvalidValue;   // the imaging condition belongs to the adjoint
+    const cudaError_t e = G.ndim == 3 ? (T.adjoint ? tti_passes<32, 8, 16, 2, true>(G, T, s) : tti_passes<32, 8, 16, 2, false>(G, T, s))
+                                      : (T.adjoint ? tti_passes<128, 1, 1, 1, true>(G, T, s) : tti_passes<128, 1, 1, 1, false>(G, T, s));
     if (e != cudaSuccess) return e;
     count_launch(2);
     if (J.npts > 0) {
         dim3 g2((J.npts * J.ncorner + 255) / 256, T.nshots);
-        tti_inject_kernel<<<g2, 256, 0, s>>>(G, T, J.idx, J.w, J.npts, J.ncorner, J.traces, J.tr_ss,
-                                             J.tr_ts, J.tr_rs, J.step, J.sign, J.both);
+        pdl_launch(tti_inject_kernel, g2, 256, 0, s, G, T, J.idx, J.w, J.npts, J.ncorner, J.traces, J.tr_ss, J.tr_ts,
+                   J.tr_rs, J.step, J.sign, J.both);
         count_launch();
     }
     prof_end(PROF_STENCIL, ev, s);

@@ -279,6 +279,10 @@ Layout make_layout(const wp_model_s *M, const wp_geom *g, int r, int Tb, int mod
     const int nparts = residual_parts((long long)S * nt * g->nrec);
     L.partials = c.take<double>(nparts);
     L.misfit = c.take<double>(1);
+    if (M->G.tti) {   // E, S and dt^2/m one after the other: one tensor map covers them (tti.cu)
+        L.E = c.take<float>(NP);
+        L.Sd = c.take<float>(NP);
+    }
     L.b = c.take<float>(NP);
     const size_t ki = inj_ints(M->G, S);
     L.t.src_off = c.take<int>(ki);
@@ -299,8 +303,6 @@ Layout make_layout(const wp_model_s *M, const wp_geom *g, int r, int Tb, int mod
     if (M->G.tti) {
         L.t.s_idx = c.take<int>(std::max<size_t>(1, (size_t)S * g->nsrc * nc));
         L.t.s_w = c.take<float>(std::max<size_t>(1, (size_t)S * g->nsrc * nc));
-        L.E = c.take<float>(NP);
-        L.Sd = c.take<float>(NP);
         L.ax = c.take<float>(NP);
         L.ay = c.take<float>(NP);
         L.az = c.take<float>(NP);
@@ -672,23 +674,18 @@ cudaError_t validation_resources(float **scratch, cudaStream_t *stream)
     return cudaSuccess;
 }
 
-// Planes marched by one stencil block.  Short marches give more blocks (about eight waves
-// of resident blocks balance the uneven blocks: injection, absorbing layers, the ragged
-// last segment, the prologue latency); long marches amortise the 8-plane z halo, so the
-// march is kept >= 24 planes where the grid allows.
+// Planes marched by one single-step block: each segment reads its 8-plane z halo again, and a
+// plane time grows with the load (choose_segment).  Measured in 3-D: 12 planes on a padded 144^3
+// (26.8 us a step with its contraction; 29.5 at the former least of 24), within 1 % of the best
+// on 208^3, 336^3 and 592 x 592 x 336 (flat from 34 to 112 planes).
 int choose_tz(const GridDev &G, int nshots)
 {
     if (const char *e = getenv("WP_STENCIL_TZ")) {
         const int v = atoi(e);
         if (v >= 1) return std::min(v, G.NZ);
     }
-    const long long cols = (long long)tiles_x(G) * tiles_y(G) * nshots;
-    const long long cap = (long long)device_sm_count() * stencil_blocks_per_sm(G);
-    const long long segs = std::max<long long>(1, (8 * cap + cols - 1) / cols);
-    int tz = (int)((G.NZ + segs - 1) / segs);
-    tz = std::max(tz, std::min(24, G.NZ));
-    const int nseg = (G.NZ + tz - 1) / tz;
-    return (G.NZ + nseg - 1) / nseg;   // equal segments
+    return choose_segment(G.NZ, (double)tiles_x(G) * tiles_y(G) * nshots,
+                          (double)device_sm_count() * stencil_blocks_per_sm(G), 2.0 * RAD);
 }
 
 // Planes per two-step segment (2-D isotropic grids; 0 turns two-step launches off).  A launch

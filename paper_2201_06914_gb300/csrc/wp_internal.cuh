@@ -302,6 +302,24 @@ int stencil_blocks_per_sm(const GridDev &G);
 cudaError_t launch_stencil2(const GridDev &G, const StencilArgs &A, cudaStream_t s);
 int stencil2_blocks_per_sm(const GridDev &G);
 int device_sm_count();
+// Planes per z segment of a march whose blocks cover `cols` tile columns (all shots), `cap`
+// resident blocks on the device, `extra` planes of start-up per segment: minimises
+// (tz + extra) (1 + f) with f = blocks / cap, a lone block's plane time plus one that grows in
+// proportion to the load; equal segments.
+inline int choose_segment(int NZ, double cols, double cap, double extra)
+{
+    int best = NZ;
+    double cost = 1e300;
+    for (int nseg = 1; nseg <= NZ; nseg++) {
+        const int tz = (NZ + nseg - 1) / nseg;
+        const double c = (tz + extra) * (1.0 + cols * ((NZ + tz - 1) / tz) / cap);
+        if (c < cost) {
+            cost = c;
+            best = tz;
+        }
+    }
+    return best;
+}
 cudaError_t launch_gather(const GridDev &G, const StencilArgs &A, cudaStream_t s);
 cudaError_t launch_probe_gemm(const GemmArgs &A, int nshots, cudaStream_t s);
 cudaError_t launch_probe_split(const float *Q, int nshots, int nt, int r, int r_pad, int nt_pad,
@@ -460,6 +478,9 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
+
+// The line at p into L2.
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // 16-byte asynchronous copy global -> shared; `bytes` = 0 writes zeros (the address is
 // still a valid one).
