@@ -134,8 +134,10 @@ double wp_model_vmax(const wp_model_t *model);
  * wp_adjoint_image reads and writes, and wp_offset_image reads (Eq. 3, Eq. 4), chosen per
  * model handle (the default is WP_PROBES_DENSE):
  *   WP_PROBES_DENSE    row (shot, probe) holds the model's N points, x fastest; rows are N
- *                      floats apart.  The library accumulates in the aligned layout and
- *                      copies into this one once per call (one read and one write of P).
+ *                      floats apart.  Where the padded NX is a multiple of 4 the library
+ *                      writes these rows directly; otherwise it accumulates in the aligned
+ *                      layout and copies into this one once per call (one read and one
+ *                      write of P).
  *   WP_PROBES_ALIGNED  rows are row_floats floats apart (N_aligned rounded up to 128, so
  *                      every row starts on a 512-byte boundary) and point (x, y, z) of a
  *                      row sits at ((z * NY + y) * x_pitch + x), where x_pitch is the padded

@@ -595,7 +595,8 @@ static cudaError_t launch_probe_pipe_slice(const PipeArgs &A, int nshots, cudaSt
     dim3 grid((unsigned)std::min<long long>(items, g_num_sms));
     cudaEvent_t ev = prof_begin(PROF_GEMM, s);
     PipeMaps TM = ring_maps(A, nshots);
-    if (A.ntiles * 128LL > A.P_pitch || !p_map(A, nshots, psl, &TM.pmap)) return cudaErrorInvalidValue;
+    // (a tile past the end of a row is clipped by the tensor map)
+    if (A.Np > A.P_pitch || !p_map(A, nshots, psl, &TM.pmap)) return cudaErrorInvalidValue;
     kern<<<grid, PIPE_THREADS, smem, s>>>(A, PL, nshots, TM);
     prof_end(PROF_GEMM, ev, s);
     count_launch();
@@ -669,11 +670,12 @@ __global__ void probe_dot_kernel(const float *__restrict__ Pu, bool pu_aligned, 
     }
 }
 
-// Both operands row-aligned: one thread per 4 consecutive points of a row (16-byte loads of
+// Both operands at x pitch NXp with rows `upitch` and `vpitch` floats apart (multiples of 4: the
+// row-aligned layout, or dense rows of a grid whose NX is a multiple of 4): one thread per 4 consecutive points of a row (16-byte loads of
 // both operands; rows of NXp points, a multiple of 4), the same per-point summation order
 // as probe_dot_kernel, so the image is bitwise the same.
-__global__ void probe_dot4_kernel(const float *__restrict__ Pu, const float *__restrict__ Pv, long long rows,
-                                  int NX, int NXp, long long pitch, int r, int nshots, float scale,
+__global__ void probe_dot4_kernel(const float *__restrict__ Pu, long long upitch, const float *__restrict__ Pv,
+                                  long long vpitch, long long rows, int NX, int NXp, int r, int nshots, float scale,
                                   float *__restrict__ g)
 {
     const int q4 = NXp / 4;
@@ -684,13 +686,13 @@ __global__ void probe_dot4_kernel(const float *__restrict__ Pu, const float *__r
         const long long w = row * NXp + x;
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         for (int sh = 0; sh < nshots; sh++) {
-            const float *a = Pu + (long long)sh * r * pitch + w;
-            const float *b = Pv + (long long)sh * r * pitch + w;
+            const float *a = Pu + (long long)sh * r * upitch + w;
+            const float *b = Pv + (long long)sh * r * vpitch + w;
             float part[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
             for (int i = 0; i < r; i++) {
-                const float4 av = __ldg((const float4 *)(a + (long long)i * pitch));
-                const float4 bv = __ldg((const float4 *)(b + (long long)i * pitch));
+                const float4 av = __ldg((const float4 *)(a + (long long)i * upitch));
+                const float4 bv = __ldg((const float4 *)(b + (long long)i * vpitch));
                 part[0] = fmaf(av.x, bv.x, part[0]);
                 part[1] = fmaf(av.y, bv.y, part[1]);
                 part[2] = fmaf(av.z, bv.z, part[2]);
@@ -706,18 +708,20 @@ __global__ void probe_dot4_kernel(const float *__restrict__ Pu, const float *__r
     }
 }
 
-cudaError_t launch_probe_dot(const float *Pu, bool pu_aligned, const float *Pv, long long N, int NX, int NXp,
-                             long long pitch, int r, int nshots, float scale, float *g, cudaStream_t s)
+cudaError_t launch_probe_dot(const float *Pu, bool pu_aligned, const float *Pv, long long vpitch, long long N, int NX,
+                             int NXp, long long pitch, int r, int nshots, float scale, float *g, cudaStream_t s)
 {
-    if (pu_aligned && (NXp & 3) == 0 && (pitch & 3) == 0 && !((uintptr_t)Pu & 15) && !((uintptr_t)Pv & 15)) {
+    const long long upitch = pu_aligned ? pitch : N;
+    if ((pu_aligned || NX == NXp) && (NXp & 3) == 0 && (upitch & 3) == 0 && (vpitch & 3) == 0 && !((uintptr_t)Pu & 15) &&
+        !((uintptr_t)Pv & 15)) {
         const long long rows = N / NX, work = rows * (NXp / 4);
         const long long blocks = std::min<long long>((work + 255) / 256, 152LL * 64);
-        probe_dot4_kernel<<<(unsigned)blocks, 256, 0, s>>>(Pu, Pv, rows, NX, NXp, pitch, r, nshots, scale, g);
+        probe_dot4_kernel<<<(unsigned)blocks, 256, 0, s>>>(Pu, upitch, Pv, vpitch, rows, NX, NXp, r, nshots, scale, g);
         count_launch();
         return cudaGetLastError();
     }
     const long long blocks = std::min<long long>((N + 255) / 256, 152LL * 64);
-    probe_dot_kernel<<<(unsigned)blocks, 256, 0, s>>>(Pu, pu_aligned, Pv, N, NX, NXp, pitch, r, nshots, scale, g);
+    probe_dot_kernel<<<(unsigned)blocks, 256, 0, s>>>(Pu, pu_aligned, Pv, N, NX, NXp, vpitch, r, nshots, scale, g);
     count_launch();
     return cudaGetLastError();
 }

@@ -339,11 +339,11 @@ cudaError_t launch_offset_image(const float *Pu, const float *Pv, bool aligned, 
                                 cudaStream_t s);
 // Device address of the offset kernels' error flag (static device memory).
 cudaError_t offset_err_ptr(int **p);
-// g[u] = scale * sum_s sum_i Pu[s][i][.] * Pv[s][i][w(u)]: Pv in the row-aligned layout
-// (rows of `pitch` floats, point u at w(u) = row * NXp + x), Pu dense (rows of N, at u) or,
-// with pu_aligned, in the same layout as Pv
-cudaError_t launch_probe_dot(const float *Pu, bool pu_aligned, const float *Pv, long long N, int NX, int NXp,
-                             long long pitch, int r, int nshots, float scale, float *g, cudaStream_t s);
+// g[u] = scale * sum_s sum_i Pu[s][i][.] * Pv[s][i][w(u)]: Pv with rows of `vpitch` floats and
+// point u at w(u) = row * NXp + x, Pu dense (rows of N, at u) or, with pu_aligned, rows of `pitch`
+// floats with u at w(u)
+cudaError_t launch_probe_dot(const float *Pu, bool pu_aligned, const float *Pv, long long vpitch, long long N, int NX,
+                             int NXp, long long pitch, int r, int nshots, float scale, float *g, cudaStream_t s);
 // row-aligned probe rows -> dense layout
 cudaError_t launch_p_to_user(const float *in, long long pitch, long long rows, long long N, int NX,
                              int NXp, float *out, cudaStream_t s);
