@@ -128,21 +128,17 @@ extern "C" wp_status wp_probe_accumulate_static(const float *A, int cnt, long lo
     // The array keeps the previous call's contents: the error flag must start at zero.
     e = cudaMemsetAsync(err, 0, 256, s);
     if (e != cudaSuccess) return static_fail(WP_ERR_CUDA, "clearing the error flag failed", e);
-    e = wp::launch_probe_split(Q, nshots, nt, r, r_pad, nt_pad, qhi, qlo, s);
-    if (e != cudaSuccess) return static_fail(WP_ERR_CUDA, "probe split launch failed", e);
+    e = wp::launch_probe_images(Q, nshots, nt, r, r_pad, t0, cnt, 1, qhi, qlo, err + 32, s);
+    if (e != cudaSuccess) return static_fail(WP_ERR_CUDA, "probe image launch failed", e);
     wp::GemmArgs G{};
-    G.ring = A;
-    G.ring_ss = (long long)cnt * npoints;
-    G.nslots = cnt;
+    G.a = A;
+    G.a_ss = (long long)cnt * npoints;
     G.N = npoints;
-    G.t0 = t0;
     G.cnt = cnt;
-    G.slot0 = 0;
-    G.mode = 0;
-    G.qhi = qhi;
-    G.qlo = qlo;
-    G.q_ss = (long long)r_pad * nt_pad;
-    G.nt_pad = nt_pad;
+    G.img_hi = qhi;
+    G.img_lo = qlo;
+    G.img_ld = (long long)r_pad * 64;
+    G.lo_nz = err + 32;
     G.r = r;
     G.r_pad = r_pad;
     G.P = P;

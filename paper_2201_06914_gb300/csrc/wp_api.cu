@@ -1248,11 +1248,11 @@ wp_status wp_probe_accumulate(const float *A, int cnt, long long npoints, int ns
     __nv_bfloat16 *qhi = c.take<__nv_bfloat16>((size_t)nshots * rp * ntp);
     __nv_bfloat16 *qlo = c.take<__nv_bfloat16>((size_t)nshots * rp * ntp);
     WP_CUDA(cudaMemsetAsync(err, 0, 64 * sizeof(int), s));
+    WP_CUDA(launch_probe_images(Q, nshots, nt, r, rp, t0, cnt, 1, qhi, qlo, err + 32, s));
     if (npoints % 128 == 0) {
         // Rows of A are 512-byte aligned: use the pipelined bulk-copy kernel.
-        WP_CUDA(launch_probe_images(Q, nshots, nt, r, rp, t0, cnt, 1, qhi, qlo, err + 32, s));
         PipeArgs P{};
-            P.ring = A;
+        P.ring = A;
         P.ring_ss = (long long)cnt * npoints;
         P.sstride = npoints;
         P.nslots = cnt;
@@ -1282,22 +1282,17 @@ wp_status wp_probe_accumulate(const float *A, int cnt, long long npoints, int ns
         WP_CUDA(launch_probe_pipe(P, nshots, s));
         return WP_OK;
     }
-    WP_CUDA(launch_probe_split(Q, nshots, nt, r, rp, ntp, qhi, qlo, s));
     // this kernel keeps at most 256 probes in tensor memory: one launch per slice of 256
     for (int i0 = 0; i0 < r; i0 += 256) {
         GemmArgs G{};
-        G.ring = A;
-        G.ring_ss = (long long)cnt * npoints;
-        G.nslots = cnt;
+        G.a = A;
+        G.a_ss = (long long)cnt * npoints;
         G.N = npoints;
-        G.t0 = t0;
         G.cnt = cnt;
-        G.slot0 = 0;
-        G.mode = 0;
-        G.qhi = qhi + (long long)i0 * ntp;
-        G.qlo = qlo + (long long)i0 * ntp;
-        G.q_ss = (long long)rp * ntp;
-        G.nt_pad = ntp;
+        G.img_hi = qhi + (long long)i0 * 64;
+        G.img_lo = qlo + (long long)i0 * 64;
+        G.img_ld = (long long)rp * 64;
+        G.lo_nz = err + 32;
         G.r = std::min(256, r - i0);
         G.r_pad = std::min(256, rp - i0);
         G.P = P + (long long)i0 * npoints;
@@ -1361,11 +1356,10 @@ wp_status wp_range_finder(const float *D, int nt, int ncols, int nshots, int d_s
     WP_CUDA(cudaMemcpyAsync(L.Y, Z, (size_t)nshots * nt * r * sizeof(float), cudaMemcpyDeviceToDevice, s));
     WP_CUDA(launch_transpose(D, dss, nt, ncols, d_shared ? 1 : nshots, L.Dt, dss, s));
     GemmArgs G{};
-    G.t0 = 0;
-    G.slot0 = 0;
-    G.mode = 0;
-    G.qhi = L.qhi;
-    G.qlo = L.qlo;
+    G.img_hi = L.qhi;
+    G.img_lo = L.qlo;
+    G.img_ld = (long long)rp * 64;
+    G.lo_nz = L.err + 32;   // once a probe operand has had a lo part, it stays set
     G.r = r;
     G.r_pad = rp;
     G.scale = 1.f;
@@ -1373,28 +1367,22 @@ wp_status wp_range_finder(const float *D, int nt, int ncols, int nshots, int d_s
     for (int k = 0; k < power; k++) {
         // T = D^T Y: rows t of D are the contraction's steps, its columns the points
         WP_CUDA(cudaMemsetAsync(L.T, 0, (size_t)nshots * r * ncols * sizeof(float), s));
-        WP_CUDA(launch_probe_split(L.Y, nshots, nt, r, rp, nt_pad_of(nt), L.qhi, L.qlo, s));
-        G.ring = D;
-        G.ring_ss = dss;
-        G.nslots = nt;
+        WP_CUDA(launch_probe_images(L.Y, nshots, nt, r, rp, 0, nt, 1, L.qhi, L.qlo, L.err + 32, s));
+        G.a = D;
+        G.a_ss = dss;
         G.N = ncols;
         G.cnt = nt;
-        G.q_ss = (long long)rp * nt_pad_of(nt);
-        G.nt_pad = nt_pad_of(nt);
         G.P = L.T;
         G.P_ss = (long long)r * ncols;
         WP_CUDA(launch_probe_gemm(G, nshots, s));
         // Y = D T, as Y^T = contraction of D^T (rows c) with T^T
         WP_CUDA(launch_transpose(L.T, (long long)r * ncols, r, ncols, nshots, L.Tt, (long long)ncols * r, s));
         WP_CUDA(cudaMemsetAsync(L.Yt, 0, (size_t)nshots * r * nt * sizeof(float), s));
-        WP_CUDA(launch_probe_split(L.Tt, nshots, ncols, r, rp, nt_pad_of(ncols), L.qhi, L.qlo, s));
-        G.ring = L.Dt;
-        G.ring_ss = dss;
-        G.nslots = ncols;
+        WP_CUDA(launch_probe_images(L.Tt, nshots, ncols, r, rp, 0, ncols, 1, L.qhi, L.qlo, L.err + 32, s));
+        G.a = L.Dt;
+        G.a_ss = dss;
         G.N = nt;
         G.cnt = ncols;
-        G.q_ss = (long long)rp * nt_pad_of(ncols);
-        G.nt_pad = nt_pad_of(ncols);
         G.P = L.Yt;
         G.P_ss = (long long)r * nt;
         WP_CUDA(launch_probe_gemm(G, nshots, s));

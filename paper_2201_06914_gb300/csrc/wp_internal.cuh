@@ -251,19 +251,15 @@ inline int stencil2_seg_reach(const GridDev &G) { return 1 + (2 * RAD + G.tz2 - 
 inline int stencil2_tiles(const GridDev &G) { return tiles2_x(G) * tiles2_z(G); }
 inline long long stencil2_keys(const GridDev &G) { return (long long)stencil2_tiles(G) * (G.tz2 + 2 * RAD); }
 
-// Probe contraction arguments.
+// Probe contraction of rows of any alignment (probe_gemm.cu).
 struct GemmArgs {
-    const float *ring; long long ring_ss; int nslots; long long N;
-    int t0, cnt;     // absolute first time index of the block (probe row), valid steps
-    int slot0;       // ring slot holding step t0 (forward: increment t0)
-    int mode;        // 0: A_t = ring[slot(t)]; 1: A_t = cp*ring[slot(t+1)] - cm*ring[slot(t)]
-    const __nv_bfloat16 *qhi, *qlo; long long q_ss; int nt_pad; // [shot][r_pad][nt_pad]
-    int r, r_pad;
+    const float *a; long long a_ss; long long N; int cnt;   // [shot][cnt][N] (shot stride a_ss)
+    // swizzled probe images [shot][chunk] of one block, img_ld elements apart, and the flag
+    // launch_probe_images writes (a slice of the probes starts 64 elements per probe further)
+    const __nv_bfloat16 *img_hi, *img_lo; long long img_ld; const int *lo_nz;
+    int r, r_pad;    // r_pad <= 256
     float *P; long long P_ss;   // [shot][r][N] accumulated in place
     float scale;
-    // fused imaging after the last block: img[p] = img_scale * sum_i Pu[i][p] * P[i][p]
-    const float *Pu; long long Pu_ss; float *img; long long img_ss; float img_scale; int do_img;
-    GridDev G;
     int *err;
 };
 
@@ -322,8 +318,6 @@ inline int choose_segment(int NZ, double cols, double cap, double extra)
 }
 cudaError_t launch_gather(const GridDev &G, const StencilArgs &A, cudaStream_t s);
 cudaError_t launch_probe_gemm(const GemmArgs &A, int nshots, cudaStream_t s);
-cudaError_t launch_probe_split(const float *Q, int nshots, int nt, int r, int r_pad, int nt_pad,
-                               __nv_bfloat16 *qhi, __nv_bfloat16 *qlo, cudaStream_t s);
 cudaError_t launch_probe_pipe(const PipeArgs &A, int nshots, cudaStream_t s);
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                     const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
