@@ -10,13 +10,13 @@
 // (1-sigma dt/2)u^{n-1} = a^n.  L is the 8th-order Laplacian evaluated in difference
 // form, sum_k c_k ((u[+k] - u[0]) + (u[-k] - u[0])), with zero values beyond the grid.
 //
-// Data movement: a block owns a tile of (x, y) columns (2-D: 512 x 1, 3-D: 64 x 8; every
+// Data movement: a block owns a tile of (x, y) columns (2-D: 256 or 128 x 1, 3-D: 32 x 16; every
 // thread owns 4 adjacent columns as one float4) and marches `tz` planes along z.  Planes
 // are staged through shared memory with 16-byte cp.async copies that zero-fill outside the
-// grid (the Dirichlet exterior costs nothing): a ring holds the u tiles of planes z-4 .. z+4
+// grid (the Dirichlet exterior costs nothing): a ring holds the u tiles of planes z .. z+4
 // with their x/y halos plus LA planes in flight, a second ring the increment and dt^2/m of
-// the plane being updated.  Internal fields use a row pitch NXp (NX rounded up to 4) so
-// that every float4 is 16-byte aligned; the padding columns are kept at zero.
+// the planes being updated.  Internal fields use a row pitch NXp (NX rounded up to 4) so
+// that every float4 is 16-byte aligned; the padding columns stay zero (dt^2/m is zero there).
 //
 // Fused into the same launch:
 //   - injection of point sources (forward) or of the receiver residual (adjoint): each
@@ -27,13 +27,13 @@
 //   - the exact imaging condition of Eq. 2 (template flag IMG): g += u_tt^j * v^j with
 //     u_tt^j rebuilt from two stored forward increments.
 #include <cstdlib>
+#include <type_traits>
 
 #include "stencil_step.cuh"
 
 namespace wp {
 
 using step::P4;
-
 
 // Block = TXT x TY threads; thread (lx, ly) owns the 4 adjacent columns
 // x = x0 + 4*lx + j (j < 4) of row y = y0 + ly, so a tile is TX = 4*TXT columns wide.  The
@@ -42,57 +42,46 @@ using step::P4;
 // Along z every thread keeps its own float4 of the nine planes z-4 .. z+4 in registers
 // (the march loop is unrolled by U planes and the window slides by U once per group).
 // Shared memory only serves the neighbours inside a plane: a ring of NU u tiles with x/y
-// halos, filled with 16-byte cp.async copies that zero-fill outside the grid (the Dirichlet
-// exterior costs nothing), and a ring of NDB tiles holding the increment and dt^2/m of the
-// planes being updated.  LA planes are in flight; one barrier per plane.
-#ifndef WP_STENCIL_U
-#define WP_STENCIL_U 3
-#endif
-#ifndef WP_STENCIL_LA3D
-#define WP_STENCIL_LA3D 3
-#endif
-// NA: fields staged per plane in the increment ring (2: the increment and dt^2/m; 5 for the
-// 2-D exact-imaging variant, which also stages the two history rows and the image it updates,
-// so that their loads do not sit in the step's critical path).
-template <int TXT, int TY, int NA = 2>
+// halos, and a ring of NDB tiles holding the increment and dt^2/m of the planes being updated.
+// LA planes are in flight; one barrier per plane.
+//
+// What bounds it: in 3-D the 20 B a point and step through HBM (512 x 512 x 256 padded by 40: 410 us
+// a step = 5.74 TB/s; 450 us before) and the instruction latency of 12 warps a SM; so, as in the
+// two-step kernel, every shared-memory access has a constant offset from one of two registers,
+// every global one is a multiply-add from one offset, nothing outside the grid is tested and
+// groups without injection entries run a copy of the loop without the lookups (174 instructions
+// per 128 points, 270 before).  32 x 16 tiles read 1.9 floats of u per point instead of the 2.25
+// of 64 x 8 and waste fewer columns on rows that are no multiple of 64.  Four blocks a SM at 128
+// registers take 414 us.
+template <int TXT, int TY>
 struct StencilShape {
     static constexpr int TX = 4 * TXT;
     static constexpr int HY = TY > 1 ? RAD : 0;
     static constexpr int NT = TXT * TY;
     static constexpr int W = TX + 2 * RAD;
     static constexpr int H = TY + 2 * HY;
-    static constexpr int U = WP_STENCIL_U;           // planes per unrolled group
-    static constexpr int LA = TY > 1 ? WP_STENCIL_LA3D : 3;   // planes in flight: u z+5.., db z+1..
-    static constexpr int NU = 8;                     // u ring: planes z .. z+4+LA
-    static constexpr int NDB = 4;                    // increment/model ring
+    static constexpr int U = 4;                      // planes per unrolled group
+    static constexpr int LA = 3;                     // planes in flight: u z+5.., db z+1..
+    static constexpr int NU = 8;                     // u ring (two groups): planes z .. z+4+LA
+    static constexpr int NDB = 4;                    // increment/model ring (one group)
     static constexpr int USLOT = H * W;              // floats
-    static constexpr int DBSLOT = NA * TY * TX;      // floats
+    static constexpr int DBSLOT = 2 * TY * TX;       // floats
     static constexpr int UCH = USLOT / 4;            // 16-byte chunks per u tile
-    static constexpr int DBCH = DBSLOT / 4;
     static constexpr int UK = (UCH + NT - 1) / NT;   // u chunks per thread
-    static constexpr int DK = (DBCH + NT - 1) / NT;  // increment/model chunks per thread
     static constexpr size_t SMEM = (size_t)(NU * USLOT + NDB * DBSLOT) * sizeof(float);
     // resident blocks per SM (launch bound: 2-D registers <= 128; 3-D <= 168, the y
     // neighbours add 32 live registers)
     static constexpr int MINB = TY > 1 ? 3 : 8192 / (NT * 16) > 16 ? 16 : 8192 / (NT * 16);
-    static_assert(RAD + 1 + LA <= NU && LA + 1 <= NDB, "rings");
-    static_assert((NU & (NU - 1)) == 0 && (NDB & (NDB - 1)) == 0, "ring sizes are powers of two");
+    static_assert(NU == 2 * U && NDB == U && U == RAD && RAD + 1 + LA <= NU && LA + 1 <= NDB, "rings");
 };
 
-template <int TXT, int TY, bool IMG>
-constexpr int stencil_na() { return (IMG && TY == 1) ? 5 : 2; }
-
 template <int TXT, int TY, bool IMG, bool WD>
-__global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT, TY, IMG>()>::MINB)
-    stencil_kernel(const GridDev G, const StencilArgs A)
+__global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY>::MINB) stencil_kernel(const GridDev G, const StencilArgs A)
 {
-    using S = StencilShape<TXT, TY, stencil_na<TXT, TY, IMG>()>;
-    constexpr int TX = S::TX, HY = S::HY, W = S::W, NT = S::NT, LA = S::LA, U = S::U;
-    constexpr int NU = S::NU, NDB = S::NDB;
-    constexpr uint32_t USZ = S::USLOT * 4, DSZ = S::DBSLOT * 4;   // slot bytes
+    using S = StencilShape<TXT, TY>;
+    constexpr int TX = S::TX, HY = S::HY, W = S::W, NT = S::NT, LA = S::LA, U = S::U, NU = S::NU, NDB = S::NDB;
+    constexpr uint32_t USZ = S::USLOT * 4, DSZ = S::DBSLOT * 4, OB = TY * TX * 4;   // slot bytes; dt^2/m in a slot
     extern __shared__ float4 smem4[];
-    float *uring = (float *)smem4;
-    float *dbring = uring + NU * S::USLOT;
     __shared__ float sq[TY][TX];
     __shared__ int inj_lo, inj_hi;
     __shared__ step::f2 coef[8];
@@ -111,12 +100,16 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
     const int x0 = (tile % ntx) * TX, y0 = ((tile / ntx) % nty) * TY;
     const int z0 = (tile / (ntx * nty)) * G.tz, z1 = min(z0 + G.tz, G.NZ);
     const int nplanes = z1 - z0;
-    const int NXp = G.NXp, PS = G.NXp * G.NY;
+    const int NXp = G.NXp, PS = G.NXp * G.NY, NZ = G.NZ;
     const float *__restrict__ u = A.u_in + sh * A.u_in_ss;
+    const int gy = y0 + ly, xc = x0 + 4 * lx;
+    const bool row_ok = gy < G.NY && xc < NXp;   // this thread's float4 lies in the field
+    const int own = row_ok ? gy * NXp + xc : 0;
 
-    // Copy descriptors of this thread (fixed across planes): shared-memory byte offset,
-    // global address at plane 0 (a valid address even for chunks outside the grid in x/y,
-    // which copy 0 bytes and so zero-fill).
+    // Copies of this thread (fixed across planes): shared-memory byte offset, global address at
+    // plane 0 (a valid one even for chunks outside the grid in x/y, which copy 0 bytes and so
+    // zero-fill).  The increment and dt^2/m are only read by the thread that copies them.
+    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(smem4);
     uint32_t us[S::UK];
     const float *ug[S::UK];
     int un16[S::UK];
@@ -127,58 +120,41 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
         const int x = x0 - RAD + 4 * k4, y = y0 - HY + r;
         const bool v = c < S::UCH && x >= 0 && x < NXp && y >= 0 && y < G.NY;
         un16[k] = v ? 16 : 0;
-        us[k] = (uint32_t)(r * W + 4 * k4) * 4;
+        us[k] = sb + (uint32_t)(r * W + 4 * k4) * 4;
         ug[k] = u + (v ? y * NXp + x : 0);
     }
-    uint32_t ds[S::DK];
-    const float *dg[S::DK];
-    int dn16[S::DK];
+    const uint32_t sd = sb + NU * USZ + 16u * tid;
+    const int nd = row_ok ? 16 : 0;
+    const float *gd = A.d_in + sh * A.d_in_ss + own, *gb = A.b + own;
+    const int ulim = min(NZ, z1 + RAD);
+    // u plane k (zeros beyond the grid and the segment) into the slot at byte offset o of the ring
+    auto issue_u = [&](int k, int ko, uint32_t o) {
+        if (k < ulim) {
 #pragma unroll
-    for (int k = 0; k < S::DK; k++) {
-        const int c = tid + k * NT;
-        const int a = c / (TY * TX / 4), rem = c % (TY * TX / 4);
-        const int r = rem / (TX / 4), k4 = rem % (TX / 4);
-        const int x = x0 + 4 * k4, y = y0 + r;
-        const bool v = c < S::DBCH && x < NXp && y < G.NY;
-        dn16[k] = v ? 16 : 0;
-        ds[k] = (uint32_t)(a * TY * TX + r * TX + 4 * k4) * 4;
-        const float *src = a == 0 ? A.d_in + sh * A.d_in_ss
-                         : a == 1 ? A.b
-                         : a == 2 ? A.h1 + sh * A.h_ss
-                         : a == 3 ? A.h0 + sh * A.h_ss
-                                  : A.img + sh * A.img_ss;
-        dg[k] = src + (v ? y * NXp + x : 0);
-    }
-    const uint32_t su0 = (uint32_t)__cvta_generic_to_shared(uring);
-    const uint32_t sd0 = (uint32_t)__cvta_generic_to_shared(dbring);
-    // u plane k (< NZ) into ring slot (k - z0) mod NU; planes beyond the grid are never read
-    auto issue_u = [&](int k) {
-        if (k >= G.NZ) return;
-        const uint32_t base = su0 + (uint32_t)((k - z0) & (NU - 1)) * USZ;
-        const long long ko = (long long)k * PS;
+            for (int q = 0; q < S::UK; q++)
+                if ((q + 1) * NT <= S::UCH || tid + q * NT < S::UCH) cp_async16(us[q] + o, ug[q] + ko, un16[q]);
+        } else {
 #pragma unroll
-        for (int q = 0; q < S::UK; q++)
-            if ((q + 1) * NT <= S::UCH || tid + q * NT < S::UCH) cp_async16(base + us[q], ug[q] + ko, un16[q]);
+            for (int q = 0; q < S::UK; q++)
+                if ((q + 1) * NT <= S::UCH || tid + q * NT < S::UCH) step::sts(us[q] + o, step::zero());
+        }
     };
-    // increment/model plane k (< z1) into ring slot (k - z0) mod NDB
-    auto issue_db = [&](int k) {
+    // increment/model plane k (< z1) into ring slot
+    auto issue_db = [&](int k, int ko, int slot) {
         if (k >= z1) return;
-        const uint32_t base = sd0 + (uint32_t)((k - z0) & (NDB - 1)) * DSZ;
-        const long long ko = (long long)k * PS;
-#pragma unroll
-        for (int q = 0; q < S::DK; q++)
-            if ((q + 1) * NT <= S::DBCH || tid + q * NT < S::DBCH) cp_async16(base + ds[q], dg[q] + ko, dn16[q]);
+        cp_async16(sd + slot * DSZ, gd + ko, nd);
+        cp_async16(sd + slot * DSZ + OB, gb + ko, nd);
     };
 
     // Prologue.  Group g < LA holds u plane z0+4+g and db plane z0+g; group 0 also holds
     // the u planes z0 .. z0+3.  Planes z0-4 .. z0-1 are only needed in the window and are
     // read straight from global memory.
 #pragma unroll
-    for (int k = 0; k < RAD; k++) issue_u(z0 + k);
+    for (int k = 0; k < RAD; k++) issue_u(z0 + k, (z0 + k) * PS, k * USZ);
 #pragma unroll
     for (int g = 0; g < LA; g++) {
-        issue_u(z0 + RAD + g);
-        issue_db(z0 + g);
+        issue_u(z0 + RAD + g, (z0 + RAD + g) * PS, (RAD + g) * USZ);
+        issue_db(z0 + g, (z0 + g) * PS, g);
         cp_async_commit();
     }
     // March indices with injection entries (sources or receivers in this tile).
@@ -199,17 +175,15 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
             }
 
     const float *tr = tile_inj ? A.traces + sh * A.tr_ss + (long long)A.step * A.tr_ts : nullptr;
-    const int gy = y0 + ly, xc = x0 + 4 * lx;
-    const bool row_ok = gy < G.NY && xc < NXp;   // this thread's float4 lies in the field
     float sdx[4];
 #pragma unroll
     for (int j = 0; j < 4; j++)
         sdx[j] = damp_term(xc + j, G.nx, G.nbl, G.hs0x, G.inv_nbl) +
                  (TY > 1 ? damp_term(gy, G.ny, G.nbl, G.hs0y, G.inv_nbl) : 0.f);
-    // all four columns outside the x (and y) absorbing layers
-    const bool col_int = sdx[0] == 0.f && sdx[1] == 0.f && sdx[2] == 0.f && sdx[3] == 0.f;
-    const bool has_pad = xc + 4 > G.NX;          // some of the 4 columns are row padding
-    const long long own = (long long)gy * NXp + xc;
+    // the whole warp outside the x (and y) absorbing layers (points outside the grid do not matter)
+    const bool warp_int =
+        __all_sync(0xffffffffu, !row_ok || (sdx[0] == 0.f && sdx[1] == 0.f && sdx[2] == 0.f && sdx[3] == 0.f));
+    const int zs0 = G.nbl, zs1 = G.nbl + G.nz;   // planes outside the z absorbing layers
     float *uo = A.u_out + sh * A.u_out_ss + own;
     float *dout = A.d_out + sh * A.d_out_ss + own;
 
@@ -220,52 +194,64 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
         const int zz = z0 - RAD + k;
         win[k] = (row_ok && zz >= 0) ? *(const P4 *)(u + (long long)zz * PS + own) : step::zero();
     }
-    const uint32_t ub = su0 + (uint32_t)((ly + HY) * W * 4) + (uint32_t)(RAD + 4 * lx) * 4;
-    const uint32_t db = sd0 + (uint32_t)((ly * TX + 4 * lx) * 4);
+    const uint32_t ub = sb + (uint32_t)((ly + HY) * W * 4) + (uint32_t)(RAD + 4 * lx) * 4;   // own float4 in a u tile
     cp_async_wait<LA - 1>();
     __syncthreads();
-    const int zlo = inj_lo, zhi = inj_hi;
+    const int klo = inj_lo, khi = inj_hi;
     const step::Coef K = step::coef_load(&coef);
 #pragma unroll
-    for (int k = 0; k < RAD; k++) win[RAD + k] = (z0 + k < G.NZ) ? step::lds(ub + (uint32_t)k * USZ) : step::zero();
+    for (int k = 0; k < RAD; k++) win[RAD + k] = step::lds(ub + (uint32_t)k * USZ);
 
-    const int zs0 = G.nbl, zs1 = G.nbl + G.nz;   // planes outside the z absorbing layers
     const int warp = tid >> 5, lane = tid & 31;
-    for (int zb = z0; zb < z1; zb += U) {
+    // u slot s of the ring: groups of four planes start at slot 0 or 4, so slot s < 4 is at f0 + s USZ
+    // and slot s >= 4 at f1 + s USZ, f0 = f1 = 0 in even groups, f0 = 4 USZ and f1 = -4 USZ in odd ones
+    uint32_t f0 = 0, f1 = 0, flip = U * USZ;
+    int kz = z0 * PS;
 #pragma unroll
-        for (int ph = 0; ph < U; ph++) {
-            const int z = zb + ph;
-            if (z >= z1) break;
-            const int rel = z - z0;
-            cp_async_wait<LA - 1>();
-            __syncthreads();
-            issue_u(z + RAD + LA);
-            issue_db(z + LA);
-            cp_async_commit();
-
-            win[2 * RAD + ph] = (z + RAD < G.NZ) ? step::lds(ub + (uint32_t)((rel + RAD) & (NU - 1)) * USZ)
-                                                 : step::zero();   // plane z+4
-            const uint32_t az = ub + (uint32_t)(rel & (NU - 1)) * USZ;
-            const P4 wl = step::lds(az - 16);
-            const P4 wr = step::lds(az + 16);
-            P4 yp[RAD], ym[RAD];
-            if (TY > 1) {
+    for (int q = 0; q < S::UK; q++) ug[q] += (RAD + LA) * (long long)PS;
+    gd += LA * (long long)PS;
+    gb += LA * (long long)PS;
+    // plane z = group start + PH; INJ: a source or receiver may lie in it
+    auto plane = [&](auto phc, auto injc, int z) {
+        constexpr int PH = decltype(phc)::value;
+        constexpr bool INJ = decltype(injc)::value;
+        auto slot = [&](auto sc) -> uint32_t {
+            constexpr int q = decltype(sc)::value & (NU - 1);
+            return (q < U ? f0 : f1) + q * USZ;
+        };
+        cp_async_wait<LA - 1>();
+        __syncthreads();
+        issue_u(z + RAD + LA, kz, slot(std::integral_constant<int, PH + RAD + LA>{}));
+        issue_db(z + LA, kz, (PH + LA) & (NDB - 1));
+        cp_async_commit();
+        if (IMG && row_ok && z + 2 < z1) {   // the history rows and the image two planes ahead, into L2
+            const long long p = kz + 2 * (long long)PS + own;
+            prefetch_l2(A.h1 + sh * A.h_ss + p);
+            prefetch_l2(A.h0 + sh * A.h_ss + p);
+            prefetch_l2(A.img + sh * A.img_ss + p);
+        }
+        const uint32_t az = ub + slot(std::integral_constant<int, PH>{});
+        win[2 * RAD + PH] = step::lds(ub + slot(std::integral_constant<int, PH + RAD>{}));   // plane z+4
+        const P4 wl = step::lds(az - 16), wr = step::lds(az + 16);
+        P4 yp[RAD], ym[RAD];
+        if (TY > 1) {
 #pragma unroll
-                for (int k = 1; k <= RAD; k++) {
-                    yp[k - 1] = step::lds(az + (uint32_t)(k * W * 4));
-                    ym[k - 1] = step::lds(az - (uint32_t)(k * W * 4));
-                }
+            for (int k = 1; k <= RAD; k++) {
+                yp[k - 1] = step::lds(az + (uint32_t)(k * W * 4));
+                ym[k - 1] = step::lds(az - (uint32_t)(k * W * 4));
             }
-            const uint32_t adb = db + (uint32_t)(rel & (NDB - 1)) * DSZ;
-            const P4 din = step::lds(adb);
-            const P4 bb = step::lds(adb + TY * TX * 4);
+        }
+        const P4 din = step::lds(sd + PH * DSZ), bb = step::lds(sd + PH * DSZ + OB);
 
+        bool inj = false;
+        if (INJ) {
+            const int rel = z - z0;
             int e0 = 0, e1 = 0;
-            if (rel >= zlo && rel <= zhi) {
+            if (rel >= klo && rel <= khi) {
                 e0 = off[key0 + rel];
                 e1 = off[key0 + rel + 1];
             }
-            const bool inj = e1 > e0;
+            inj = e1 > e0;
             if (inj) {
                 // each warp sums the entries of its own columns: entry column a belongs to
                 // thread (a / TX) * TXT + (a % TX) / 4, so no block barrier is needed
@@ -278,31 +264,23 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
                 }
                 __syncwarp();
             }
-            if (!row_ok) continue;
-            P4 dn, un;
-            float sdv[4];
-            step::step4<(TY > 1), WD>(&win[ph], yp, ym, wl, wr, din, bb, &sq[ly][4 * lx], inj,
-                                  col_int && z >= zs0 && z < zs1, sdx, z, G, K, dn, un, sdv);
-            if (has_pad) step::zero_pad(xc, G.NX, dn, un);   // padding columns stay zero
-            const long long oz = (long long)z * PS;
-            *(P4 *)(uo + oz) = un;
-            *(P4 *)(dout + oz) = dn;
+        }
+        P4 dn, un;
+        float sdv[4];
+        step::step4<(TY > 1), WD>(&win[PH], yp, ym, wl, wr, din, bb, &sq[ly][4 * lx], inj,
+                                  warp_int && z >= zs0 && z < zs1, sdx, z, G, K, dn, un, sdv);
+        if (row_ok) {
+            *(P4 *)(uo + kz) = un;
+            *(P4 *)(dout + kz) = dn;
             if (IMG) {
                 float u4[4];
                 step::upk(un.a, u4[0], u4[1]);
                 step::upk(un.b, u4[2], u4[3]);
-                const long long p = oz + own;
-                float4 h1, h0, gv;
+                const long long p = (long long)kz + own;
                 float4 *gi = (float4 *)(A.img + sh * A.img_ss + p);
-                if (S::DBSLOT == 5 * TY * TX) {   // staged with the increment (2-D)
-                    h1 = *(const float4 *)&dbring[(rel & (NDB - 1)) * S::DBSLOT + 2 * TY * TX + ly * TX + 4 * lx];
-                    h0 = *(const float4 *)&dbring[(rel & (NDB - 1)) * S::DBSLOT + 3 * TY * TX + ly * TX + 4 * lx];
-                    gv = *(const float4 *)&dbring[(rel & (NDB - 1)) * S::DBSLOT + 4 * TY * TX + ly * TX + 4 * lx];
-                } else {
-                    h1 = *(const float4 *)(A.h1 + sh * A.h_ss + p);
-                    h0 = *(const float4 *)(A.h0 + sh * A.h_ss + p);
-                    gv = *gi;
-                }
+                const float4 h1 = *(const float4 *)(A.h1 + sh * A.h_ss + p);
+                const float4 h0 = *(const float4 *)(A.h0 + sh * A.h_ss + p);
+                float4 gv = *gi;
                 gv.x += A.img_scale * ((1.f + sdv[0]) * h1.x - (1.f - sdv[0]) * h0.x) * u4[0];
                 gv.y += A.img_scale * ((1.f + sdv[1]) * h1.y - (1.f - sdv[1]) * h0.y) * u4[1];
                 gv.z += A.img_scale * ((1.f + sdv[2]) * h1.z - (1.f - sdv[2]) * h0.z) * u4[2];
@@ -310,9 +288,23 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY, stencil_na<TXT,
                 *gi = gv;
             }
         }
+        kz += PS;
+    };
+    auto group = [&](auto injc, int zb) {
+        plane(std::integral_constant<int, 0>{}, injc, zb);
+        if (zb + 1 < z1) plane(std::integral_constant<int, 1>{}, injc, zb + 1);
+        if (zb + 2 < z1) plane(std::integral_constant<int, 2>{}, injc, zb + 2);
+        if (zb + 3 < z1) plane(std::integral_constant<int, 3>{}, injc, zb + 3);
+    };
+    for (int zb = z0; zb < z1; zb += U) {
+        if (klo < zb - z0 + U && khi >= zb - z0) group(std::true_type{}, zb);
+        else group(std::false_type{}, zb);
         // slide the window by U planes
 #pragma unroll
         for (int k = 0; k < 2 * RAD; k++) win[k] = win[k + U];
+        f0 += flip;
+        f1 -= flip;
+        flip = 0u - flip;
     }
     cp_async_wait<0>();
 }
@@ -322,7 +314,7 @@ __global__ void gather_kernel(const StencilArgs A) { gather_rows(A, blockIdx.x);
 template <int TXT, int TY, bool IMG, bool WD>
 static void launch_variant(const GridDev &G, const StencilArgs &A, dim3 grid, cudaStream_t s)
 {
-    using S = StencilShape<TXT, TY, stencil_na<TXT, TY, IMG>()>;
+    using S = StencilShape<TXT, TY>;
     cudaFuncSetAttribute(stencil_kernel<TXT, TY, IMG, WD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     pdl_launch(stencil_kernel<TXT, TY, IMG, WD>, grid, S::NT, S::SMEM, s, G, A);
 }

@@ -687,8 +687,8 @@ cudaError_t validation_resources(float **scratch, cudaStream_t *stream)
 
 // Planes marched by one single-step block: each segment reads its 8-plane z halo again, and a
 // plane time grows with the load (choose_segment).  Measured in 3-D: 12 planes on a padded 144^3
-// (26.8 us a step with its contraction; 29.5 at the former least of 24), within 1 % of the best
-// on 208^3, 336^3 and 592 x 592 x 336 (flat from 34 to 112 planes).
+// (26.8 us a step with its contraction; 29.5 at the former least of 24), within 2 % of the best
+// on 208^3, 336^3 and 592 x 592 x 336 (403 .. 417 us from 34 to 112 planes, 458 at 168).
 int choose_tz(const GridDev &G, int nshots)
 {
     if (const char *e = getenv("WP_STENCIL_TZ")) {

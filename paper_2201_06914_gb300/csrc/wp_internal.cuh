@@ -76,9 +76,9 @@ struct InjEntry {
 // the host and stored in GridDev::tx and GridDev::tz).
 // Each thread owns 4 adjacent columns (one float4), so a tile is (4 * threads_x) x TY.
 //   2-D: TY = 1, TX = 128 (32 threads) or 256 (64 threads), whichever pads NX less;
-//   3-D: 16 x 8 threads, 64 x 8 columns.
+//   3-D: 8 x 16 threads, 32 x 16 columns.
 constexpr int T2Y = 1;
-constexpr int T3TX = 16, T3X = 4 * T3TX, T3Y = 8;
+constexpr int T3TX = 8, T3X = 4 * T3TX, T3Y = 16;
 constexpr int RAD = 4;                               // stencil radius (space order 8)
 
 struct StencilArgs {
