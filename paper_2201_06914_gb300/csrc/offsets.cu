@@ -303,12 +303,14 @@ __global__ void __launch_bounds__(OT_THREADS, 1) offset_tc_kernel(const OffArgs 
 // 1 KB each), so the split is done in place: every converter reads its share of a half into
 // registers, the converters meet at a barrier, and each writes its hi and lo chunks.  With
 // no separate staging area, two full stages fit, so a chunk's copies land while the
-// previous chunk is converted and multiplied:
-//   warp 12      producer: three tiled TMA copies per 64-k chunk into stage j mod 2 once
+// previous chunk is converted and multiplied (what bounds it: copy, conversion and MMAs of a chunk
+// in turn over two stages; 81 offsets of 16 shots x 64 probes on 1681 x 481: 2.66 ms, 2.85 ms with
+// eight converter warps that tested every value against the row ends):
+//   warp 20      producer: three tiled TMA copies per 64-k chunk into stage j mod 2 once
 //                the MMAs of chunk j - 2 have released it;
-//   warps 0-7    converters: per half, read (k, 8 points) units, zero the points outside
+//   warps 0-15   converters: per half, read (k, 8 points) units, zero the points outside
 //                the x-row, barrier, write hi / lo;
-//   warps 8-11   epilogue as in offset_tc_kernel; lane 0 of warp 8 issues the MMAs with
+//   warps 16-19  epilogue as in offset_tc_kernel; lane 0 of warp 16 issues the MMAs with
 //                MN-major ("transposed") A and B descriptors.
 // Atom addresses (bytes from the stage; kg = k / 8 within the chunk, mi / ni = point / 64,
 // hl = 0 for hi, 1 for lo):
@@ -316,9 +318,11 @@ __global__ void __launch_bounds__(OT_THREADS, 1) offset_tc_kernel(const OffArgs 
 //   B: 32768 + hl * 256 NBh + kg * 16 NBp + ni * 1024 (box hl's FP32 rows of 4 NBh bytes)
 // so half h of A covers [16384 h, +16384) and half h of box b covers 32768 + 256 NBh b +
 // [128 NBh h, +128 NBh) in both views.
-constexpr int MN_THREADS = 416;   // warps 0-7 converters, 8-11 epilogue + MMA issue, 12 producer
-constexpr int MN_WPROD = 12;
-constexpr int MN_UNITS = 7;       // (k, 8-point) units per converter thread and half (NBp <= 320)
+constexpr int MN_CONV = 512;                     // converter threads
+constexpr int MN_EPI = MN_CONV / 32;             // first epilogue warp (MMA issue in its lane 0)
+constexpr int MN_WPROD = MN_EPI + 4;
+constexpr int MN_THREADS = 32 * (MN_WPROD + 1);
+constexpr int MN_UNITS = 1792 / MN_CONV + (1792 % MN_CONV != 0);   // (k, 8-point) units per converter and half (NBp <= 320)
 
 __host__ __device__ inline int mn_nbp(int NB) { return (NB + 63) / 64 * 64; }
 __host__ __device__ inline uint32_t mn_stage_bytes(int NBp) { return 32768u + (uint32_t)NBp * 256u; }
@@ -336,7 +340,7 @@ __device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo,
     return d;
 }
 
-__global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_constant__ OffMaps TM)
+__global__ void __maxnreg__(80) offset_mn_kernel(const OffArgs A, const __grid_constant__ OffMaps TM)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // a shared pointer
@@ -356,7 +360,7 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
     if (tid == 0) {
         for (int s = 0; s < 2; s++) {
             mbar_init(&fbar[s], 1);
-            mbar_init(&full[s], OCONV);
+            mbar_init(&full[s], MN_CONV);
             mbar_init(&empty[s], 1);
         }
         mbar_init(&accfull, 1);
@@ -364,7 +368,7 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
         abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp == OW_EPI) tmem_alloc(&tmem_holder, ncols);
+    if (warp == MN_EPI) tmem_alloc(&tmem_holder, ncols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -396,7 +400,7 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
                 if (issued >= 1) mbar_wait_bounded(&fbar[(issued - 1) & 1], (uint32_t)(((issued - 1) >> 1) & 1));
             }
         }
-    } else if (warp < OW_EPI) {
+    } else if (warp < MN_EPI) {
         // ---------------- converters ----------------
         // Unit u < 512: A, k row u / 16 of the half, points 8 (u % 16) .. +7; u >= 512: box
         // b of B, k row and 8-point group from the remainder.  Offsets (bytes from the stage)
@@ -410,7 +414,7 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
         bool isb[MN_UNITS];
 #pragma unroll
         for (int i = 0; i < MN_UNITS; i++) {
-            const int u = tid + OCONV * i;
+            const int u = tid + MN_CONV * i;
             xr[i] = -0x40000000;
             isb[i] = false;
             src[i] = dst[i] = 0;
@@ -435,8 +439,9 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
             const long long row = item / A.ntx;
             const int a0 = (int)(item - row * A.ntx) * 128, b0 = a0 - A.boff;
             const bool got = mbar_wait_abortable(&fbar[s], (uint32_t)((j >> 1) & 1), &abort_flag);
-            if (bar_any<1, OCONV>(!got)) break;
+            if (bar_any<1, MN_CONV>(!got)) break;
             const uint32_t st = smem_u32(stage_ptr(s));
+            const bool inside = b0 >= 0 && b0 + NBp <= A.NX && a0 + 128 <= A.NX;   // of the whole item
 #pragma unroll
             for (int h = 0; h < 2; h++) {
                 float v[MN_UNITS][8];
@@ -451,12 +456,14 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
                                  : "=f"(q1.x), "=f"(q1.y), "=f"(q1.z), "=f"(q1.w) : "r"(a + 16));
                     v[i][0] = q0.x; v[i][1] = q0.y; v[i][2] = q0.z; v[i][3] = q0.w;
                     v[i][4] = q1.x; v[i][5] = q1.y; v[i][6] = q1.z; v[i][7] = q1.w;
-                    const int x = (isb[i] ? b0 : a0) + xr[i];
+                    if (!inside) {
+                        const int x = (isb[i] ? b0 : a0) + xr[i];
 #pragma unroll
-                    for (int e = 0; e < 8; e++)
-                        if (x + e < 0 || x + e >= A.NX) v[i][e] = 0.f;   // outside the x-row
+                        for (int e = 0; e < 8; e++)
+                            if (x + e < 0 || x + e >= A.NX) v[i][e] = 0.f;   // outside the x-row
+                    }
                 }
-                asm volatile("bar.sync 3, %0;" ::"n"(OCONV) : "memory");   // half h read by all
+                asm volatile("bar.sync 3, %0;" ::"n"(MN_CONV) : "memory");   // half h read by all
 #pragma unroll
                 for (int i = 0; i < MN_UNITS; i++) {
                     if (xr[i] == -0x40000000) continue;
@@ -475,8 +482,8 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
             mbar_arrive(&full[s]);
         }
     } else {
-        // ---------------- epilogue (warps 8-11), MMA issue in lane 0 of warp 8 ----------------
-        const int ew = warp - OW_EPI;
+        // ---------------- epilogue (warps 16-19), MMA issue in lane 0 of warp 16 ----------------
+        const int ew = warp - MN_EPI;
         const int N1 = NBp < 256 ? NBp : 256, N2 = NBp - N1;
         constexpr uint32_t MNMAJ = (1u << 15) | (1u << 16);   // A and B MN-major
         const uint32_t id1 = idesc_bf16_f32(128, N1) | MNMAJ, id2 = N2 > 0 ? (idesc_bf16_f32(128, N2) | MNMAJ) : 0u;
@@ -551,7 +558,7 @@ __global__ void __maxnreg__(128) offset_mn_kernel(const OffArgs A, const __grid_
 
     __syncthreads();
     if (abort_flag && tid == 0) atomicExch(A.err, 4);
-    if (warp == OW_EPI) {
+    if (warp == MN_EPI) {
         tc_fence_after();
         tmem_dealloc(tmem, ncols);
     }
