@@ -130,22 +130,20 @@ extern "C" wp_status wp_probe_accumulate_static(const float *A, int cnt, long lo
     if (e != cudaSuccess) return static_fail(WP_ERR_CUDA, "clearing the error flag failed", e);
     e = wp::launch_probe_images(Q, nshots, nt, r, r_pad, t0, cnt, 1, qhi, qlo, err + 32, s);
     if (e != cudaSuccess) return static_fail(WP_ERR_CUDA, "probe image launch failed", e);
-    wp::GemmArgs G{};
+    wp::RowsArgs G{};
     G.a = A;
     G.a_ss = (long long)cnt * npoints;
     G.N = npoints;
     G.cnt = cnt;
     G.img_hi = qhi;
     G.img_lo = qlo;
-    G.img_ld = (long long)r_pad * 64;
     G.lo_nz = err + 32;
     G.r = r;
     G.r_pad = r_pad;
     G.P = P;
-    G.P_ss = (long long)r * npoints;
     G.scale = scale;
     G.err = err;
-    e = wp::launch_probe_gemm(G, nshots, s);
+    e = wp::launch_probe_rows(G, nshots, s);
     if (e != cudaSuccess) return static_fail(WP_ERR_CUDA, "probe contraction launch failed", e);
     return WP_OK;
 }

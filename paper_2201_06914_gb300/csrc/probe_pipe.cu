@@ -1,15 +1,18 @@
-// Pipelined probe accumulation on the tensor cores (Eq. 3), the hot-path version of
-// probe_gemm.cu.  For every shot and every 128-point tile of the grid:
+// Pipelined probe accumulation on the tensor cores (Eq. 3).  For every shot and every 128-point tile of the grid:
 //   P[i][x] += scale * sum_{t < cnt} A[t][x] * Q[t0 + t][i]
 // where A is read from the time-step ring (forward: u_tt rebuilt from two consecutive
-// stored increments; adjoint: the adjoint wavefield itself).
+// stored increments; adjoint: the adjoint wavefield itself) or from a caller's rows of any length
+// (wp_probe_accumulate, wp_probe_accumulate_static, the two products of the range finder).
+// Both operands are split into bfloat16 hi + lo; the four products accumulate in FP32 in tensor
+// memory, which keeps the contraction faithful to FP32 (relative error ~2^-17) for any probe
+// matrix, Rademacher or orthonormal.
 //
 // One persistent CTA per SM runs a warp-specialised pipeline over its (shot, tile) items:
 //   warp 12    producer: per 64-step chunk, one or two tiled TMA copies of the 64 (or 65)
 //              ring rows of the tile plus the pre-swizzled probe image(s) (bf16 hi, and lo
 //              unless the probes are exact bfloat16 values) into a stage of shared memory,
 //              completing on the stage's `full` mbarrier;
-//   warps 0-7  converters: one grid point and half of the chunk's steps per thread,
+//   warps 0-7  converters: one grid point per thread and all or half of the chunk's steps,
 //              FP32 -> u_tt (or v) -> bfloat16 hi + lo, written in the K-major
 //              128-byte-swizzled layout tcgen05 reads;
 //   warp 13    MMA issuer (one thread): 2 or 4 bf16 products per 16-step k-slice into the
@@ -109,7 +112,20 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
 }
+__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+        : "memory");
+}
 constexpr uint32_t A32_BYTES = 33792;     // 65 rows x 512 B, rounded to 1 KiB
+// ROWS: a chunk is four groups (residues of the row number) of 16 rows of 132 floats: the 128
+// points of the tile and the up to 3 floats by which a row starts past a 16-byte boundary
+constexpr int ROWS_W = 132;
+constexpr uint32_t ROWS_GROUP = 16 * ROWS_W * 4;
+static_assert(4 * ROWS_GROUP <= A32_BYTES, "stage");
 
 __host__ __device__ inline uint32_t pipe_cols(int r_pad)
 {
@@ -136,20 +152,6 @@ struct PipePlan {
     uint32_t stg_off;   // byte offset of the epilogue staging
 };
 constexpr int MAXST = 4;
-
-// Named barrier over the 256 converter threads that also returns, to every one of them,
-// whether any of them failed its wait: the converters leave their loops together, so no
-// thread is left waiting at the barrier for one that has gone.
-__device__ __forceinline__ bool converters_any(bool failed)
-{
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred q, p;\n\t"
-                 "setp.ne.u32 q, %1, 0;\n\t"
-                 "bar.red.or.pred p, 1, 256, q;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(r) : "r"((uint32_t)failed) : "memory");
-    return r != 0;
-}
 
 // try_wait that lets the hardware suspend the thread for up to `ns` nanoseconds (it wakes
 // as soon as the phase completes), so waiting roles do not spin on the issue slots the
@@ -203,7 +205,10 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
 // overlaps the MMAs of the next); above, one accumulator takes all 512 columns and each
 // product is two MMAs (N = 256 and r_pad - 256, the largest N of one instruction being 256),
 // so the ring is read once for up to 512 probes.
-template <int RB, int PS>
+// ROWS: the steps are a caller's rows of any length (launch_probe_rows): four tensor maps, one per
+// residue of the row number modulo 4, cover rows that start at any 4-byte boundary, and P, whose
+// rows start anywhere too, is read and written by the epilogue's threads.
+template <int RB, int PS, bool ROWS>
 __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeArgs A, const PipePlan PL, int nshots,
                                                                      const __grid_constant__ PipeMaps TM)
 {
@@ -213,6 +218,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
     __shared__ uint32_t tmem_holder;
     __shared__ int abort_flag;
 
+    constexpr bool SPLIT = RB > 64;   // all converters on every chunk (see there)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // probes that are exact bfloat16 values (Rademacher +-1) have an all-zero lo part: its
     // image is not staged and its two products are skipped (the flag is written before this
@@ -230,7 +236,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
         for (int s = 0; s < ST; s++) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
-            mbar_init(&aready[s], NCONV);
+            mbar_init(&aready[s], SPLIT ? NCONV : NCONV / 2);
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(&accfull[b], 1);
@@ -261,9 +267,17 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
                 const int need = A.cnt - c * CH;
                 const int rows = A.mode ? min(CH + 1, need + 1) : min(CH, need);
                 uint8_t *st = stage_ptr(s);
-                if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)(rows * 512 + (qlo ? 2 : 1) * img_bytes));
+                if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)((ROWS ? 4 * ROWS_GROUP : rows * 512) + (qlo ? 2 : 1) * img_bytes));
                 __syncwarp();
-                if (TM.use) {
+                if (ROWS) {
+                    // rows G0 .. G0 + 63 of the caller's matrix: sixteen of each residue, from the
+                    // first one at or after G0 (rows past the block are masked, past the end zero)
+                    if (lane < 4) {
+                        const int G0 = (A.ring_ss ? shot * A.cnt : 0) + c * CH;
+                        tma_load_2d(st + lane * ROWS_GROUP, &TM.map[lane >> 1][lane & 1], tile * 128, (G0 - lane + 3) >> 2,
+                                    &full[s]);
+                    }
+                } else if (TM.use) {
                     if (lane == 0) {
                         tma_load_3d(st, &TM.map[c][0], tile * 128, TM.slot[c][0], shot, &full[s]);
                         if (TM.rows[c][1] > 0)
@@ -345,64 +359,124 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
         }
     } else if (warp < WEPI) {
         // ---------------- converters ----------------
-        const int m = tid & 127, half = tid >> 7;   // point, steps [32 half, 32 half + 32)
+        // Up to 64 probes (four stages, a chunk's copy takes 1500 cycles) the converters are two groups of 128 threads (one point each, all 64 steps), one for the
+        // even stages and one for the odd ones, so that one group's shared-memory latencies and
+        // barrier run under the other's work: with all 256 threads on one chunk a chunk took 2000
+        // cycles of mostly waiting.  A group sees every phase of its stages' barriers (a parity
+        // wait cannot tell a phase it skipped from the one before), so chunks go to groups by
+        // stage, not by number.  Above, with three stages or fewer, all threads convert every
+        // chunk, 32 steps each (256 probes: 5.3 instead of 5.5 ms per 256-step block of 16 shots).
+        const int m = tid & 127, grp = tid >> 7;
         uint32_t g = 0;
-        // No early exit on the abort flag here: a failed wait is voted on by all converters
+        // No early exit on the abort flag here: a failed wait is voted on by the group
         for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-            const int tile = item % A.ntiles;
-            const long long p = (long long)tile * 128 + m;
-            const long long prow = div_pts(p, A.NXp, small);
-            const bool valid = p < A.Np && (int)(p - prow * A.NXp) < A.NX;
             float cp = 1.f, cm = 1.f;
-            if (A.mode == 1 && valid) {
+            if (A.mode == 1) {
+                const int tile = item % A.ntiles;
+                const long long p = (long long)tile * 128 + m;
+                const long long prow = div_pts(p, A.NXp, small);
                 const int x = (int)(p - prow * A.NXp);
                 const int z = (int)div_pts(prow, A.G.NY, small), y = (int)(prow - (long long)z * A.G.NY);
                 const float sd = damp_at(A.G, x, y, z);
                 cp = 1.f + sd;
                 cm = 1.f - sd;
             }
+            // the warp's points all lie outside the absorbing layer: u_tt is a plain difference
+            const bool inner = __all_sync(0xffffffffu, cp == 1.f);
             bool ok = true;
             for (int c = 0; c < nch; c++, g++) {
                 const int s = g % ST;
+                if (!SPLIT && (s & 1) != grp) continue;
                 const bool got = wait_bar(&full[s], (g / ST) & 1, &abort_flag);
                 uint8_t *st = stage_ptr(s);
-                const float *a32 = (const float *)st;
+                const float *col = (const float *)st + m;
                 uint8_t *ah = st;            // the operand overwrites the FP32 rows in place
                 uint8_t *al = ah + 16384;
-                const int need = A.cnt - c * CH - half * (CH / 2);   // valid steps of this half
-                const bool rd = valid && got;
-                const float *col = a32 + half * (CH / 2) * 128 + m;
-                float v[CH / 2];
-                if (A.mode == 0) {
+                const int need = A.cnt - c * CH;   // valid steps of the chunk
+                // Points beyond the grid (row padding, the last tile's end) need no mask: the ring
+                // holds zeros in the padding, the copies zero-fill past the last point, and
+                // whatever they hold reaches only their own, unspecified entries of P.  Full
+                // chunks (all but a block's last) run without a test per step.
+                constexpr int NHALF = SPLIT ? 1 : 2;   // halves of 32 steps of this thread
+                float v[NHALF][CH / 2];
 #pragma unroll
-                    for (int t = 0; t < CH / 2; t++) v[t] = (rd && t < need) ? col[t * 128] : 0.f;
-                } else {
-                    float prev = (rd && need > 0) ? col[0] : 0.f;
+                for (int i = 0; i < NHALF; i++) {
+                    const int h = SPLIT ? grp : i;
+                    const float *q = col + h * (CH / 2) * 128;
+                    const int nh = need - h * (CH / 2);
+                    if (ROWS) {
+                        // step t = 4 j + e is row j of the group of residue (G0 + e) mod 4
+                        const int G0 = (A.ring_ss ? (item / A.ntiles) * A.cnt : 0) + c * CH;
 #pragma unroll
-                    for (int t = 0; t < CH / 2; t++) {
-                        const bool in = rd && t < need;
-                        const float nx = in ? col[(t + 1) * 128] : 0.f;
-                        v[t] = in ? cp * nx - cm * prev : 0.f;
-                        prev = nx;
+                        for (int e = 0; e < 4; e++) {
+                            const int rho = (G0 + e) & 3, d = (int)((rho * (A.P_pitch & 3)) & 3);
+                            const float *qe = col + rho * (int)(ROWS_GROUP / 4) + d + h * (CH / 8) * ROWS_W;
+                            if (nh >= CH / 2) {
+#pragma unroll
+                                for (int j = 0; j < CH / 8; j++) v[i][4 * j + e] = qe[j * ROWS_W];
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < CH / 8; j++) v[i][4 * j + e] = 4 * j + e < nh ? qe[j * ROWS_W] : 0.f;
+                            }
+                        }
+                    } else if (nh >= CH / 2) {
+                        if (A.mode == 0) {
+#pragma unroll
+                            for (int t = 0; t < CH / 2; t++) v[i][t] = q[t * 128];
+                        } else {
+                            float prev = q[0];
+                            if (inner) {
+#pragma unroll
+                                for (int t = 0; t < CH / 2; t++) {
+                                    const float nx = q[(t + 1) * 128];
+                                    v[i][t] = nx - prev;
+                                    prev = nx;
+                                }
+                            } else {
+#pragma unroll
+                                for (int t = 0; t < CH / 2; t++) {
+                                    const float nx = q[(t + 1) * 128];
+                                    v[i][t] = cp * nx - cm * prev;
+                                    prev = nx;
+                                }
+                            }
+                        }
+                    } else if (A.mode == 0) {
+#pragma unroll
+                        for (int t = 0; t < CH / 2; t++) v[i][t] = t < nh ? q[t * 128] : 0.f;
+                    } else {
+                        float prev = nh > 0 ? q[0] : 0.f;
+#pragma unroll
+                        for (int t = 0; t < CH / 2; t++) {
+                            const float nx = t < nh ? q[(t + 1) * 128] : 0.f;
+                            v[i][t] = t < nh ? cp * nx - cm * prev : 0.f;
+                            prev = nx;
+                        }
                     }
                 }
-                // every converter has read its FP32 column before any operand byte is written
-                if (converters_any(!got)) {
+                // the chunk's threads have read their FP32 columns before any operand byte is written
+                const bool bad = SPLIT ? bar_any<1, NCONV>(!got)
+                               : grp == 0 ? bar_any<1, NCONV / 2>(!got) : bar_any<3, NCONV / 2>(!got);
+                if (bad) {
                     ok = false;
                     break;
                 }
 #pragma unroll
-                for (int c4 = 0; c4 < 4; c4++) {
-                    const int cc = half * 4 + c4;   // 16-byte chunk = 8 steps of the row
-                    const uint32_t off = (uint32_t)m * 128u + ((uint32_t)(cc ^ (m & 7)) << 4);
-                    const float *x = v + c4 * 8;
-                    uint4 h, l;
-                    split2(x[0], x[1], h.x, l.x);
-                    split2(x[2], x[3], h.y, l.y);
-                    split2(x[4], x[5], h.z, l.z);
-                    split2(x[6], x[7], h.w, l.w);
-                    *(uint4 *)(ah + off) = h;
-                    *(uint4 *)(al + off) = l;
+                for (int i = 0; i < NHALF; i++) {
+                    const int h = SPLIT ? grp : i;
+#pragma unroll
+                    for (int c4 = 0; c4 < 4; c4++) {
+                        const int cc = h * 4 + c4;   // 16-byte chunk = 8 steps of the row
+                        const uint32_t off = (uint32_t)m * 128u + ((uint32_t)(cc ^ (m & 7)) << 4);
+                        const float *x = v[i] + c4 * 8;
+                        uint4 hi, lo;
+                        split2(x[0], x[1], hi.x, lo.x);
+                        split2(x[2], x[3], hi.y, lo.y);
+                        split2(x[4], x[5], hi.z, lo.z);
+                        split2(x[6], x[7], hi.w, lo.w);
+                        *(uint4 *)(ah + off) = hi;
+                        *(uint4 *)(al + off) = lo;
+                    }
                 }
                 fence_proxy_async_smem();
                 mbar_arrive(&aready[s]);
@@ -421,10 +495,43 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
         for (int item = blockIdx.x; item < nitems; item += gridDim.x, j++) {
             const int shot = item / A.ntiles, tile = item % A.ntiles;
             const uint32_t ab = nacc == 2 ? (j & 1) : 0u, aph = nacc == 2 ? ((j >> 1) & 1) : (j & 1);
+            const uint32_t taddr = tmem + ab * ncols + ((uint32_t)(ew * 32) << 16);
+            if (ROWS) {
+                // one point per thread; P of the first 32 probes is read before the wait for the
+                // accumulator, of the next 32 while these are written
+                const long long p = (long long)tile * 128 + e;
+                const bool valid = p < A.N;
+                float *P = A.P + (long long)shot * A.P_ss + (valid ? p : 0);
+                bool bad = false;
+                for (int c0 = 0; c0 < A.r_pad; c0 += 32) {
+                    float old[32];
+#pragma unroll
+                    for (int i = 0; i < 32; i++) old[i] = (valid && c0 + i < A.r) ? P[(long long)(c0 + i) * A.P_pitch] : 0.f;
+                    if (c0 == 0) {
+                        const bool ok = wait_bar(&accfull[ab], aph, &abort_flag);
+                        bad = epi_any(!ok);
+                        if (bad) break;
+                        tc_fence_after();
+                    }
+#pragma unroll
+                    for (int i = 0; i < 32; i += 16) {
+                        if (c0 + i >= A.r_pad) continue;
+                        uint32_t r16[16];
+                        tmem_ld16(taddr + (uint32_t)(c0 + i), r16);
+#pragma unroll
+                        for (int q = 0; q < 16; q++)
+                            if (valid && c0 + i + q < A.r)
+                                P[(long long)(c0 + i + q) * A.P_pitch] = fmaf(A.scale, __uint_as_float(r16[q]), old[i + q]);
+                    }
+                }
+                if (bad) break;
+                tc_fence_before();
+                mbar_arrive(&accempty[ab]);
+                continue;
+            }
             const bool ok = wait_bar(&accfull[ab], aph, &abort_flag);
             if (epi_any(!ok)) break;
             tc_fence_after();
-            const uint32_t taddr = tmem + ab * ncols + ((uint32_t)(ew * 32) << 16);
 #pragma unroll
             for (int c0 = 0; c0 < RB; c0 += PS) {
                 if (c0 < A.r_pad) {
@@ -575,7 +682,7 @@ static cudaError_t launch_probe_pipe_slice(const PipeArgs &A, int nshots, cudaSt
     for (int lo = 0; lo < 2; lo++) {
         PL.sb[lo] = stage_bytes(A.r_pad, lo != 0);
         PL.st[lo] = (int)std::min<size_t>(MAXST, avail / PL.sb[lo]);
-        if (PL.st[lo] < 1) return cudaErrorInvalidValue;
+        if (PL.st[lo] < (rb <= 64 ? 2 : 1)) return cudaErrorInvalidValue;   // two converter groups need two stages
     }
     // Deeper pipelines measured slower once P's traffic is large (4 instead of 3 stages at
     // 128 probes, 3 instead of 2 at 256: 5-6 % longer), so without the lo image the plan
@@ -584,10 +691,10 @@ static cudaError_t launch_probe_pipe_slice(const PipeArgs &A, int nshots, cudaSt
     PL.st[0] = std::min(PL.st[0], std::max(PL.st[1], 2));
     PL.stg_off = std::max((uint32_t)PL.st[0] * PL.sb[0], (uint32_t)PL.st[1] * PL.sb[1]);
     const size_t smem = (size_t)PL.stg_off + pbytes + 1024;
-    auto kern = rb == 16 ? probe_pipe_kernel<16, PSL> : rb == 32 ? probe_pipe_kernel<32, 16>
-              : rb == 64 ? probe_pipe_kernel<64, 16> : rb == 128 ? probe_pipe_kernel<128, 16>
-              : rb == 256 ? probe_pipe_kernel<256, 16>
-              : psl == 32 ? probe_pipe_kernel<512, 32> : probe_pipe_kernel<512, 16>;
+    auto kern = rb == 16 ? probe_pipe_kernel<16, PSL, false> : rb == 32 ? probe_pipe_kernel<32, 16, false>
+              : rb == 64 ? probe_pipe_kernel<64, 16, false> : rb == 128 ? probe_pipe_kernel<128, 16, false>
+              : rb == 256 ? probe_pipe_kernel<256, 16, false>
+              : psl == 32 ? probe_pipe_kernel<512, 32, false> : probe_pipe_kernel<512, 16, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long items = (long long)A.ntiles * nshots;
@@ -601,6 +708,85 @@ static cudaError_t launch_probe_pipe_slice(const PipeArgs &A, int nshots, cudaSt
     prof_end(PROF_GEMM, ev, s);
     count_launch();
     return cudaGetLastError();
+}
+
+// Tensor maps of points [x0, x0 + n) of a caller's rows of N floats, `nrows` of them one after the
+// other: residue rho's map starts at row rho, rounded down to a 16-byte boundary, and its rows are
+// 4 N floats (a multiple of 16 bytes whatever N is) apart; a row ends at its own end, so nothing
+// past the matrix is read.
+static bool rows_maps(const RowsArgs &A, long long nrows, long long x0, long long n, PipeMaps *TM)
+{
+    encode_tiled_fn enc = encoder();
+    if (!enc || ((uintptr_t)A.a & 15) || nrows > 0x7fffffff) return false;
+    for (int rho = 0; rho < 4; rho++) {
+        // (a matrix of fewer than four rows: the other residues' copies are never used)
+        const bool has = rho < nrows;
+        const int d = has ? (int)((rho * (A.N & 3)) & 3) : 0;
+        const cuuint64_t dims[2] = {(cuuint64_t)(n + d), (cuuint64_t)(has ? (nrows - rho + 3) / 4 : 1)};
+        const cuuint64_t strides[1] = {(cuuint64_t)A.N * 16};
+        const cuuint32_t box[2] = {ROWS_W, 16}, estr[2] = {1, 1};
+        if (enc(&TM->map[rho >> 1][rho & 1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                (void *)(A.a + x0 + (has ? rho * A.N - d : 0)), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    return true;
+}
+
+// What bounds it: HBM (A once, P read and written) and, as in the ring's form, the converters'
+// latency.  16 shots of 281 x 281 points, 256 steps, r = 64: 344 us = 5.7 TB/s; 494 us with 4-byte
+// loads into registers by 128-thread CTAs, 939 us with an index multiply per load.
+cudaError_t launch_probe_rows(const RowsArgs &A, int nshots, cudaStream_t s)
+{
+    if (A.r_pad < 16 || A.r_pad > PIPE_MAX_R || A.r_pad % 16) return cudaErrorInvalidValue;
+    for (int i0 = 0; i0 < A.r; i0 += 256) {   // at most 256 probes at once (double-buffered accumulators)
+        PipeArgs P{};
+        P.ring_ss = A.a_ss;
+        P.NX = P.NXp = 1;   // mode 0 never looks a point's place up
+        P.cnt = A.cnt;
+        P.img_hi = A.img_hi + (long long)i0 * 64;
+        P.img_lo = A.img_lo + (long long)i0 * 64;
+        P.img_ld = (long long)A.r_pad * 64;
+        P.qlo_nz = A.lo_nz;
+        P.nblocks = 1;
+        P.ncb = (A.cnt + CH - 1) / CH;
+        P.img_div = 1;
+        P.r = std::min(256, A.r - i0);
+        P.r_pad = std::min(256, A.r_pad - i0);
+        P.P_ss = (long long)A.r * A.N;
+        P.P_pitch = A.N;
+        P.scale = A.scale;
+        P.err = A.err;
+        PipePlan PL;
+        const size_t avail = 227 * 1024 - 1024 - 256;
+        for (int lo = 0; lo < 2; lo++) {
+            PL.sb[lo] = stage_bytes(P.r_pad, lo != 0);
+            PL.st[lo] = (int)std::min<size_t>(MAXST, avail / PL.sb[lo]);
+            if (PL.st[lo] < 2) return cudaErrorInvalidValue;
+        }
+        PL.stg_off = std::max((uint32_t)PL.st[0] * PL.sb[0], (uint32_t)PL.st[1] * PL.sb[1]);
+        const size_t smem = (size_t)PL.stg_off + 1024;
+        auto kern = P.r_pad <= 64 ? probe_pipe_kernel<64, 16, true> : probe_pipe_kernel<256, 16, true>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        for (long long x0 = 0; x0 < A.N; x0 += 1LL << 30) {   // a tensor coordinate has 31 bits
+            PipeMaps TM;
+            memset(&TM, 0, sizeof TM);
+            const long long n = std::min(A.N - x0, 1LL << 30), items = (n + 127) / 128 * nshots;
+            if (items >= (1LL << 31) || !rows_maps(A, (long long)A.cnt * (A.a_ss ? nshots : 1), x0, n, &TM))
+                return cudaErrorInvalidValue;
+            P.N = P.Np = n;
+            P.ntiles = (int)((n + 127) / 128);
+            P.P = A.P + (long long)i0 * A.N + x0;
+            cudaEvent_t ev = prof_begin(PROF_GEMM, s);
+            kern<<<dim3((unsigned)std::min<long long>(items, device_sm_count())), PIPE_THREADS, smem, s>>>(P, PL, nshots, TM);
+            prof_end(PROF_GEMM, ev, s);
+            count_launch();
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
 }
 
 // Swizzled probe images.  Image (shot, b, c) holds rows i < r_pad and 64 columns k, value

@@ -4,7 +4,7 @@
 // D is an nt x ncols matrix per shot (or one shared by all shots): the shot's data
 // (ncols = receivers) or the causal convolution matrix of the source wavelet (ncols = nt),
 // the two readings of A this library offers.  The two products of each power step,
-// T = D^T Y and Y = D T, run on the tensor-core probe contraction (probe_gemm.cu); this
+// T = D^T Y and Y = D T, run on the tensor-core probe contraction (probe_pipe.cu); this
 // file holds what is left: a tiled transpose and a thin QR by classical Gram-Schmidt with
 // one full reorthogonalisation (CGS2) in FP64, one cluster of CTAs per shot.  CGS2 gives Q orthonormal
 // to working precision for any numerically full-rank Y and the positive diagonal of R

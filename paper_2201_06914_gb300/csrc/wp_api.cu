@@ -1,6 +1,6 @@
 // C ABI of libwp.so (include/wp.h): validation, workspace carving, acquisition tables and
 // the time loops of the probed (Eq. 3) and exact (Eq. 2) gradients.  All device work runs
-// in the kernels of stencil.cu, probe_gemm.cu and aux.cu; this file only orchestrates.
+// in the kernels of the other files; this file only orchestrates.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -1282,25 +1282,20 @@ wp_status wp_probe_accumulate(const float *A, int cnt, long long npoints, int ns
         WP_CUDA(launch_probe_pipe(P, nshots, s));
         return WP_OK;
     }
-    // this kernel keeps at most 256 probes in tensor memory: one launch per slice of 256
-    for (int i0 = 0; i0 < r; i0 += 256) {
-        GemmArgs G{};
-        G.a = A;
-        G.a_ss = (long long)cnt * npoints;
-        G.N = npoints;
-        G.cnt = cnt;
-        G.img_hi = qhi + (long long)i0 * 64;
-        G.img_lo = qlo + (long long)i0 * 64;
-        G.img_ld = (long long)rp * 64;
-        G.lo_nz = err + 32;
-        G.r = std::min(256, r - i0);
-        G.r_pad = std::min(256, rp - i0);
-        G.P = P + (long long)i0 * npoints;
-        G.P_ss = (long long)r * npoints;
-        G.scale = scale;
-        G.err = err;
-        WP_CUDA(launch_probe_gemm(G, nshots, s));
-    }
+    RowsArgs G{};
+    G.a = A;
+    G.a_ss = (long long)cnt * npoints;
+    G.N = npoints;
+    G.cnt = cnt;
+    G.img_hi = qhi;
+    G.img_lo = qlo;
+    G.lo_nz = err + 32;
+    G.r = r;
+    G.r_pad = rp;
+    G.P = P;
+    G.scale = scale;
+    G.err = err;
+    WP_CUDA(launch_probe_rows(G, nshots, s));
     return WP_OK;
 }
 
@@ -1355,10 +1350,9 @@ wp_status wp_range_finder(const float *D, int nt, int ncols, int nshots, int d_s
     WP_CUDA(cudaMemsetAsync(L.err, 0, 64 * sizeof(int), s));
     WP_CUDA(cudaMemcpyAsync(L.Y, Z, (size_t)nshots * nt * r * sizeof(float), cudaMemcpyDeviceToDevice, s));
     WP_CUDA(launch_transpose(D, dss, nt, ncols, d_shared ? 1 : nshots, L.Dt, dss, s));
-    GemmArgs G{};
+    RowsArgs G{};
     G.img_hi = L.qhi;
     G.img_lo = L.qlo;
-    G.img_ld = (long long)rp * 64;
     G.lo_nz = L.err + 32;   // once a probe operand has had a lo part, it stays set
     G.r = r;
     G.r_pad = rp;
@@ -1373,8 +1367,7 @@ wp_status wp_range_finder(const float *D, int nt, int ncols, int nshots, int d_s
         G.N = ncols;
         G.cnt = nt;
         G.P = L.T;
-        G.P_ss = (long long)r * ncols;
-        WP_CUDA(launch_probe_gemm(G, nshots, s));
+        WP_CUDA(launch_probe_rows(G, nshots, s));
         // Y = D T, as Y^T = contraction of D^T (rows c) with T^T
         WP_CUDA(launch_transpose(L.T, (long long)r * ncols, r, ncols, nshots, L.Tt, (long long)ncols * r, s));
         WP_CUDA(cudaMemsetAsync(L.Yt, 0, (size_t)nshots * r * nt * sizeof(float), s));
@@ -1384,8 +1377,7 @@ wp_status wp_range_finder(const float *D, int nt, int ncols, int nshots, int d_s
         G.N = nt;
         G.cnt = ncols;
         G.P = L.Yt;
-        G.P_ss = (long long)r * nt;
-        WP_CUDA(launch_probe_gemm(G, nshots, s));
+        WP_CUDA(launch_probe_rows(G, nshots, s));
         WP_CUDA(launch_cgs2_qr(L.Yt, nt, r, nshots, L.W, k + 1 == power ? Q : L.Y, L.err, s));
     }
     return WP_OK;

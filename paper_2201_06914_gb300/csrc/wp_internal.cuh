@@ -251,14 +251,13 @@ inline int stencil2_seg_reach(const GridDev &G) { return 1 + (2 * RAD + G.tz2 - 
 inline int stencil2_tiles(const GridDev &G) { return tiles2_x(G) * tiles2_z(G); }
 inline long long stencil2_keys(const GridDev &G) { return (long long)stencil2_tiles(G) * (G.tz2 + 2 * RAD); }
 
-// Probe contraction of rows of any alignment (probe_gemm.cu).
-struct GemmArgs {
-    const float *a; long long a_ss; long long N; int cnt;   // [shot][cnt][N] (shot stride a_ss)
-    // swizzled probe images [shot][chunk] of one block, img_ld elements apart, and the flag
-    // launch_probe_images writes (a slice of the probes starts 64 elements per probe further)
-    const __nv_bfloat16 *img_hi, *img_lo; long long img_ld; const int *lo_nz;
-    int r, r_pad;    // r_pad <= 256
-    float *P; long long P_ss;   // [shot][r][N] accumulated in place
+// Probe contraction of a caller's rows of any length (launch_probe_rows).
+struct RowsArgs {
+    const float *a; long long a_ss; long long N; int cnt;   // [shot][cnt][N]; a_ss = 0: one matrix for all
+    // swizzled probe images [shot][chunk][r_pad * 64] of one block, and the flag launch_probe_images writes
+    const __nv_bfloat16 *img_hi, *img_lo; const int *lo_nz;
+    int r, r_pad;    // r_pad <= 512
+    float *P;        // [shot][r][N] accumulated in place
     float scale;
     int *err;
 };
@@ -317,7 +316,8 @@ inline int choose_segment(int NZ, double cols, double cap, double extra)
     return best;
 }
 cudaError_t launch_gather(const GridDev &G, const StencilArgs &A, cudaStream_t s);
-cudaError_t launch_probe_gemm(const GemmArgs &A, int nshots, cudaStream_t s);
+// P += scale * A Q for rows of any length.
+cudaError_t launch_probe_rows(const RowsArgs &A, int nshots, cudaStream_t s);
 cudaError_t launch_probe_pipe(const PipeArgs &A, int nshots, cudaStream_t s);
 typedef CUresult (*encode_tiled_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                     const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -382,7 +382,6 @@ int prof_read(int cls, double *total_ms, long long *count);
 // Sets the thread-local message returned by wp_last_error().
 void set_last_error(const char *msg);
 long long launches();
-size_t probe_gemm_smem(int r_pad);
 
 // ---------------------------------------------------------------------------------------
 // Programmatic dependent launch: a step kernel launched with pdl_launch may start while its

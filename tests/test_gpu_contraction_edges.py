@@ -20,7 +20,9 @@ def _rel(a, b):
 
 
 @pytest.mark.parametrize("npoints,cnt,r,t0", [(1, 1, 1, 0), (127, 63, 15, 8), (129, 64, 16, 0), (255, 65, 17, 16),
-                                              (1001, 130, 64, 8), (385, 128, 256, 0), (130, 200, 300, 8), (640, 70, 33, 0)])
+                                              (1001, 130, 64, 8), (385, 128, 256, 0), (130, 200, 300, 8), (640, 70, 33, 0),
+                                              # rows of whole tiles: the pipelined kernel with 4, 3, 2 and 1 stages
+                                              (128, 1, 1, 0), (384, 200, 64, 8), (20480, 330, 128, 0), (256, 130, 300, 8)])
 @pytest.mark.parametrize("exact_bf16", [True, False])   # without and with the probes' lo part
 def test_accumulate_any_row_length(npoints, cnt, r, t0, exact_bf16):
     from paper_2201_06914_gb300 import wp

@@ -27,3 +27,24 @@ def test_pairs_match_single_steps(nx, nz, off_grid, tz):
     for k in one:
         assert np.isfinite(two[k]).all(), k
         np.testing.assert_array_equal(two[k], one[k], err_msg=k)
+
+
+@pytest.mark.parametrize("nx,ny,nz,tz", [(22, 7, 12, 3), (23, 6, 9, 1), (21, 23, 13, 1000)])
+def test_3d_tile_edges(monkeypatch, nx, ny, nz, tz):
+    """3-D tiles of 32 x 16 points: rows and y extents on, one below and one past a tile, marches of
+    one plane, three planes and the whole depth, against the FP64 oracle (tolerances as in
+    test_gpu_parity.py)."""
+    from paper_2201_06914_gb300 import wp
+    from tests.cases import close
+    from tests.test_gpu_parity import GpuRun, _oracle_probed
+    monkeypatch.setenv("WP_STENCIL_TZ", str(tz))
+    case = layered_case(ndim=3, nx=nx, ny=ny, nz=nz, nbl=5, nt=60, nshots=2, off_grid=True)
+    Q = rademacher_shots(6, 2, case.nt, 4)
+    ref = _oracle_probed(case, Q, 0.25)
+    run = GpuRun(wp, case, case.m0)
+    Pu, d = run.forward(Q)
+    g, Pv = run.adjoint(ref["res"], Q, ref["Pu"], 0.25)
+    for name, a, b, tol in (("d", d, ref["d"], 1e-5), ("Pu", Pu, ref["Pu"], 1e-5), ("Pv", Pv, ref["Pv"], 1e-5),
+                            ("g", g, ref["g"].ravel(), 1e-4)):
+        ok, err = close(a, b, tol)
+        assert ok, (name, err)
