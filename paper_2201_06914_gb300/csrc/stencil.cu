@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(TXT *TY, StencilShape<TXT, TY>::MINB) stencil_
     const int z0 = (tile / (ntx * nty)) * G.tz, z1 = min(z0 + G.tz, G.NZ);
     const int nplanes = z1 - z0;
     const int NXp = G.NXp, PS = G.NXp * G.NY, NZ = G.NZ;
-    const float *__restrict__ u = A.u_in + sh * A.u_in_ss;
+    const float *u = A.u_in + sh * A.u_in_ss;
     const int gy = y0 + ly, xc = x0 + 4 * lx;
     const bool row_ok = gy < G.NY && xc < NXp;   // this thread's float4 lies in the field
     const int own = row_ok ? gy * NXp + xc : 0;

@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel
     const int NXp = G.NXp, NZ = G.NZ;
     const int xc = x0 + 4 * lx;
     const bool a_ok = xc >= 0 && xc < NXp;               // the float4 lies inside the field
-    const float *__restrict__ u = A.u_in + sh * A.u_in_ss;
+    const float *u = A.u_in + sh * A.u_in_ss;
 
     // Staging: thread lx copies float4 lx of the u row (x0 - 4 + 4 lx; lanes 0 and 1 also the
     // two last ones) and its own float4 of the increment and of dt^2/m.  Everything outside
