@@ -442,6 +442,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
 // Bounded wait: gives up after ~2^31 clock cycles (about one second) and returns false.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity)
 {
+    if (mbar_try_wait(bar, parity)) return true;
     long long start = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (clock64() - start > (1ll << 31)) return false;
