@@ -823,10 +823,15 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY, ADJ>::NT, TY > 1 ? 4 : 7)
 // the matching correction.
 __global__ void tti_inject_kernel(const GridDev G, const TtiArgs T, const int *idx, const float *w,
                                   int npts, int ncorner, const float *traces, long long tr_ss,
-                                  long long tr_ts, long long tr_rs, int step, float sign, int both)
+                                  long long tr_ts, long long tr_rs, int step, float sign, int both,
+                                  int nblk, const StencilArgs R)
 {
     pdl_trigger();
     pdl_wait();
+    if ((int)blockIdx.x >= nblk) {   // recording of the input field
+        gather_rows(R, blockIdx.x - nblk);
+        return;
+    }
     const long long sh = blockIdx.y;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= npts * ncorner) return;
@@ -983,7 +988,7 @@ static cudaError_t tti_passes(const GridDev &G, const TtiArgs &T, cudaStream_t s
     return cudaSuccess;
 }
 
-cudaError_t launch_tti_step(const GridDev &G, const TtiArgs &T, const TtiInject &J, cudaStream_t s)
+cudaError_t launch_tti_step(const GridDev &G, const TtiArgs &T, const TtiInject &J, const StencilArgs *rec, cudaStream_t s)
 {
     cudaEvent_t ev = prof_begin(PROF_STENCIL, s);
     if (T.img && !T.adjoint) return cudaErrorInvalidValue;   // the imaging condition belongs to the adjoint
@@ -991,10 +996,13 @@ cudaError_t launch_tti_step(const GridDev &G, const TtiArgs &T, const TtiInject 
                                       : (T.adjoint ? tti_passes<128, 1, 1, true>(G, T, s) : tti_passes<128, 1, 1, false>(G, T, s));
     if (e != cudaSuccess) return e;
     count_launch(2);
-    if (J.npts > 0) {
-        dim3 g2((J.npts * J.ncorner + 255) / 256, T.nshots);
+    // Recording reads only the step's input, so it shares the injection's launch (a launch of its own,
+    // which waited for the step's end, took 2.3 of 13.0 us a step of one shot of 401 x 401).
+    const int nblk = (J.npts * J.ncorner + 255) / 256, nrec = rec ? gather_blocks(*rec, 256) : 0;
+    if (nblk + nrec > 0) {
+        dim3 g2(nblk + nrec, T.nshots);
         pdl_launch(tti_inject_kernel, g2, 256, 0, s, G, T, J.idx, J.w, J.npts, J.ncorner, J.traces, J.tr_ss, J.tr_ts,
-                   J.tr_rs, J.step, J.sign, J.both);
+                   J.tr_rs, J.step, J.sign, J.both, nblk, rec ? *rec : StencilArgs{});
         count_launch();
     }
     prof_end(PROF_STENCIL, ev, s);

@@ -482,12 +482,9 @@ wp_status launch_step(const wp_model_s *M, const wp_geom *g, const Layout &L, co
     } else {
         J.idx = L.t.g_idx; J.w = L.t.g_w; J.npts = g->nrec; J.both = 0;
     }
-    WP_CUDA(launch_tti_step(M->G, T, J, s));
-    if (A.do_gather) {
-        StencilArgs Gq = A;
-        Gq.u_in_ss = 2 * A.u_in_ss;   // record field p (virtual shot 2s)
-        WP_CUDA(launch_gather(M->G, Gq, s));
-    }
+    StencilArgs Gq = A;
+    Gq.u_in_ss = 2 * A.u_in_ss;   // record field p (virtual shot 2s)
+    WP_CUDA(launch_tti_step(M->G, T, J, A.do_gather ? &Gq : nullptr, s));
     return WP_OK;
 }
 

@@ -344,7 +344,8 @@ cudaError_t launch_p_to_user(const float *in, long long pitch, long long rows, l
 cudaError_t launch_tti_params(const GridDev &G, const float *eps, const float *delta,
                               const float *theta, const float *phi, float *E, float *Sd,
                               float *ax, float *ay, float *az, cudaStream_t s);
-cudaError_t launch_tti_step(const GridDev &G, const TtiArgs &T, const TtiInject &J, cudaStream_t s);
+// `rec` (or NULL): recording of u_in, in extra blocks of the injection's launch
+cudaError_t launch_tti_step(const GridDev &G, const TtiArgs &T, const TtiInject &J, const StencilArgs *rec, cudaStream_t s);
 cudaError_t launch_maxval(const float *x, long long n, float *out, cudaStream_t s);
 // *count += #{i : !(a[i] <= b[i]) or a value not finite} (count zeroed by the caller)
 cudaError_t launch_count_greater(const float *a, const float *b, long long n, int *count, cudaStream_t s);
