@@ -35,7 +35,8 @@
 // Measured per launch of the 1601 x 401 model (padded 1681 x 481): 64 shots 218 us (300 before;
 // 4.75 TB/s of the 20 B per point and shot it must move), 32 shots 121 (167), 16 shots 68 (94.5),
 // 8 shots 41 (57), one shot 15 (33); with the imaging condition, 16 shots: 116 us (150 before,
-// 130 without the L2 prefetch); one shot of 201 x 201: 11.2 us (39).
+// 130 without the L2 prefetch).  Launches of few blocks run stencil2_tile_kernel (below): one shot
+// of 201 x 201 4.9 us (39 before, 10.2 marching in 3-plane segments), of 401 x 401 6.5 (10.6).
 //
 // Injection uses a CSR table keyed by (tile, plane of the extended segment) that lists
 // every entry inside the extended tile (points in an overlap appear in both tiles);
@@ -72,6 +73,36 @@ struct Stencil2Shape {
     static constexpr int MINB = 384 / NT;
     static_assert(NR == 2 * U && U == RAD && RAD + 1 + LA <= NR, "rings");
 };
+
+// IMG: the imaging condition of both steps at offset o of shot sh.
+__device__ __forceinline__ void image_pair(const StencilArgs &A, long long sh, long long o, const P4 &v1, const P4 &un,
+                                           const float *sdv)
+{
+    // exact imaging of both steps at an output float4, one image read and write
+    // per launch: first u_tt of the first step (increments h2, h1) times its
+    // output v1, then that of the second (h1, h0) times un,
+    // each written as the one-step kernel writes its update, so a pair adds
+    // bit for bit what two single steps add
+    float v[4], v2[4];
+    step::upk(v1.a, v[0], v[1]);
+    step::upk(v1.b, v[2], v[3]);
+    step::upk(un.a, v2[0], v2[1]);
+    step::upk(un.b, v2[2], v2[3]);
+    float4 *gi = (float4 *)(A.img + sh * A.img_ss + o);
+    float4 gv4 = *gi;
+    const long long p = sh * A.h_ss + o;
+    const float4 h2 = *(const float4 *)(A.h2 + p), h1 = *(const float4 *)(A.h1 + p);
+    const float4 h0 = *(const float4 *)(A.h0 + p);
+    gv4.x += A.img_scale * ((1.f + sdv[0]) * h2.x - (1.f - sdv[0]) * h1.x) * v[0];
+    gv4.y += A.img_scale * ((1.f + sdv[1]) * h2.y - (1.f - sdv[1]) * h1.y) * v[1];
+    gv4.z += A.img_scale * ((1.f + sdv[2]) * h2.z - (1.f - sdv[2]) * h1.z) * v[2];
+    gv4.w += A.img_scale * ((1.f + sdv[3]) * h2.w - (1.f - sdv[3]) * h1.w) * v[3];
+    gv4.x += A.img_scale * ((1.f + sdv[0]) * h1.x - (1.f - sdv[0]) * h0.x) * v2[0];
+    gv4.y += A.img_scale * ((1.f + sdv[1]) * h1.y - (1.f - sdv[1]) * h0.y) * v2[1];
+    gv4.z += A.img_scale * ((1.f + sdv[2]) * h1.z - (1.f - sdv[2]) * h0.z) * v2[2];
+    gv4.w += A.img_scale * ((1.f + sdv[3]) * h1.w - (1.f - sdv[3]) * h0.w) * v2[3];
+    *gi = gv4;
+}
 
 template <int TXT, bool WD, bool IMG>
 __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel(const GridDev G, const StencilArgs A)
@@ -293,30 +324,7 @@ __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel
                 *(P4 *)(uo + kz) = un;
                 *(P4 *)(dout + kz) = dn;
                 if (IMG) {
-                    // exact imaging of both steps at plane rel - 4, one image read and write
-                    // per launch: first u_tt of the first step (increments h2, h1) times its
-                    // output (the window's centre), then that of the second (h1, h0) times un,
-                    // each written as the one-step kernel writes its update, so a pair adds
-                    // bit for bit what two single steps add
-                    float v[4], v2[4];
-                    step::upk(v1.a, v[0], v[1]);
-                    step::upk(v1.b, v[2], v[3]);
-                    step::upk(un.a, v2[0], v2[1]);
-                    step::upk(un.b, v2[2], v2[3]);
-                    float4 *gi = (float4 *)(A.img + sh * A.img_ss + kz + own);
-                    float4 gv4 = *gi;
-                    const long long p = sh * A.h_ss + kz + own;
-                    const float4 h2 = *(const float4 *)(A.h2 + p), h1 = *(const float4 *)(A.h1 + p);
-                    const float4 h0 = *(const float4 *)(A.h0 + p);
-                    gv4.x += A.img_scale * ((1.f + sdv[0]) * h2.x - (1.f - sdv[0]) * h1.x) * v[0];
-                    gv4.y += A.img_scale * ((1.f + sdv[1]) * h2.y - (1.f - sdv[1]) * h1.y) * v[1];
-                    gv4.z += A.img_scale * ((1.f + sdv[2]) * h2.z - (1.f - sdv[2]) * h1.z) * v[2];
-                    gv4.w += A.img_scale * ((1.f + sdv[3]) * h2.w - (1.f - sdv[3]) * h1.w) * v[3];
-                    gv4.x += A.img_scale * ((1.f + sdv[0]) * h1.x - (1.f - sdv[0]) * h0.x) * v2[0];
-                    gv4.y += A.img_scale * ((1.f + sdv[1]) * h1.y - (1.f - sdv[1]) * h0.y) * v2[1];
-                    gv4.z += A.img_scale * ((1.f + sdv[2]) * h1.z - (1.f - sdv[2]) * h0.z) * v2[2];
-                    gv4.w += A.img_scale * ((1.f + sdv[3]) * h1.w - (1.f - sdv[3]) * h0.w) * v2[3];
-                    *gi = gv4;
+                    image_pair(A, sh, kz + own, v1, un, sdv);
                 }
             }
         }
@@ -346,9 +354,159 @@ __global__ void __launch_bounds__(TXT, Stencil2Shape<TXT>::MINB) stencil2_kernel
     cp_async_wait<0>();
 }
 
+// Two steps of a small launch.  Marching fills a ring, then walks segment + 8 planes one after the
+// other; where the chip has room for the whole launch at once, the planes of a segment can run side
+// by side instead: a block holds all u^n rows of its tile in shared memory, every warp computes
+// step 1 of its plane (two planes at 256 columns) and, after one barrier, step 2.  Same tiles, same
+// keys of the injection tables and the same arithmetic as the march, so the same bits.
+// Segments have at most MAXZ planes: 16 extended planes a block (twice the segment's work in step 1,
+// in the time of one plane).  What bounds it: one latency of the L2 cache, the two steps' chains of
+// instructions and the launch; a block of 512 threads takes an SM, and further rounds of blocks cost
+// 2.7 us each, which is where the march overtakes it (choose_tz2).
+template <int TXT>
+struct Stencil2Tile {
+    static constexpr int TX = 4 * TXT, C = TX - 2 * RAD, W = TX + 2 * RAD;
+    static constexpr int NT = 512, PAR = NT / TXT;              // threads; planes side by side
+    static constexpr int MAXZ = STENCIL2_TILE_Z, PL = MAXZ + 2 * RAD, NP = PL / PAR;   // planes a thread
+    static constexpr int UR = PL + 2 * RAD;                     // u^n rows
+    static constexpr size_t SMEM = ((size_t)(UR + PL) * W + NT * 4) * sizeof(float);
+    static_assert(PL % PAR == 0, "planes");
+};
+
+template <int TXT, bool WD, bool IMG>
+__global__ void __launch_bounds__(512, 1) stencil2_tile_kernel(const GridDev G, const StencilArgs A)
+{
+    using S = Stencil2Tile<TXT>;
+    constexpr int C = S::C, W = S::W, NP = S::NP, PAR = S::PAR, TX = S::TX;
+    extern __shared__ float4 smem4[];
+    __shared__ f2 coef[8];
+    const int ntx = (G.NXp + C - 1) / C;
+    const int ntiles = ntx * ((G.NZ + G.tz2 - 1) / G.tz2);
+    if (threadIdx.x == 0) step::coef_store(&coef, G);
+    pdl_trigger();
+    pdl_wait();
+    if ((int)blockIdx.x >= ntiles) {
+        gather_rows(A, blockIdx.x - ntiles);
+        return;
+    }
+    const int lx = threadIdx.x % TXT, py = threadIdx.x / TXT, tile = blockIdx.x;
+    const long long sh = blockIdx.y;
+    const int x0 = (tile % ntx) * C - RAD;
+    const int z0 = (tile / ntx) * G.tz2, z1 = min(z0 + G.tz2, G.NZ);
+    const int zs = z0 - RAD, nrel = z1 - z0 + 2 * RAD;   // stage-A planes zs .. zs + nrel - 1
+    const int KP = G.tz2 + 2 * RAD;
+    const int NXp = G.NXp, NZ = G.NZ, xc = x0 + 4 * lx;
+    const bool a_ok = xc >= 0 && xc < NXp;
+    const float *u = A.u_in + sh * A.u_in_ss;
+    const uint32_t su = (uint32_t)__cvta_generic_to_shared(smem4), sv = su + S::UR * W * 4;   // u^n and u^{n+1} rows
+    // u^n rows of planes zs - 4 .. z1 + 7, columns x0 - 4 ..: zeros outside the grid
+    for (int c = threadIdx.x; c < (nrel + 2 * RAD) * (W / 4); c += S::NT) {
+        const int row = c / (W / 4), k = c - row * (W / 4);
+        const int x = x0 - RAD + 4 * k, z = zs - RAD + row;
+        const bool in = x >= 0 && x < NXp && z >= 0 && z < NZ;
+        cp_async16(su + 16u * c, u + (in ? z * NXp + x : 0), in ? 16 : 0);
+    }
+    cp_async_commit();
+    // own increment and dt^2/m (zeros outside the grid, where both steps then give zero)
+    P4 d[NP], b[NP];
+    const int *off = A.inj ? A.inj_off + sh * ((long long)ntiles * KP + 1) + (long long)tile * KP : nullptr;
+    int e0[NP], e1[NP];
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+        const int r = py + i * PAR, z = zs + r;
+        const bool in = r < nrel && z >= 0 && z < NZ;
+        d[i] = b[i] = step::zero();
+        e0[i] = e1[i] = 0;
+        if (in && a_ok) {
+            d[i] = *(const P4 *)(A.d_in + sh * A.d_in_ss + z * NXp + xc);
+            b[i] = *(const P4 *)(A.b + z * NXp + xc);
+        }
+        if (in && off) {
+            e0[i] = off[r];
+            e1[i] = off[r + 1];
+        }
+    }
+    const float *trA = A.inj ? A.traces + sh * A.tr_ss + (long long)A.step * A.tr_ts : nullptr;
+    const float *trB = A.inj ? A.traces + sh * A.tr_ss + (long long)A.step2 * A.tr_ts : nullptr;
+    const bool st_ok = a_ok && lx >= 1 && lx <= TXT - 2;
+    float sdx[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) sdx[j] = damp_term(xc + j, G.nx, G.nbl, G.hs0x, G.inv_nbl);
+    const bool warp_int =
+        __all_sync(0xffffffffu, !a_ok || (sdx[0] == 0.f && sdx[1] == 0.f && sdx[2] == 0.f && sdx[3] == 0.f));
+    const int ri0 = G.nbl - zs, ri1 = G.nbl + G.nz - zs;
+    const int lane = threadIdx.x & 31, half = lx >> 5;   // the warp's 128 columns of the tile
+    float *sq = (float *)smem4 + (S::UR + S::PL) * W + (threadIdx.x - lane) * 4;   // injected terms of them
+    // the terms of entries [a, e) in the warp's columns at or after lo and before hi
+    auto inject = [&](int a, int e, const float *tr, int lo, int hi) {
+        if (a >= e) return false;
+        __syncwarp();
+        *(float4 *)&sq[4 * lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncwarp();
+        for (int t = a + lane; t < e; t += 32) {
+            const InjEntry E = A.inj[t];
+            if ((E.a >> 7) == half && E.a >= lo && E.a < hi)
+                atomicAdd(&sq[E.a & 127], E.w * A.tr_sign * tr[(long long)E.trace * A.tr_rs]);
+        }
+        __syncwarp();
+        return true;
+    };
+    cp_async_wait<0>();
+    __syncthreads();
+    const step::Coef K = step::coef_load(&coef);
+    const uint32_t ou = su + 16u * lx, ov = sv + 16u * lx;
+    // ---- stage A: step 1 at every plane of the extended segment
+    P4 u1[NP];
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+        const int r = py + i * PAR;
+        if (r >= nrel) break;
+        const bool inj = inject(e0[i], e1[i], trA, 0, TX);
+        P4 w[2 * RAD + 1], dn;
+#pragma unroll
+        for (int k = 0; k <= 2 * RAD; k++) w[k] = step::lds(ou + (uint32_t)(r + k) * (W * 4) + 16);
+        const P4 al = step::lds(ou + (uint32_t)(r + RAD) * (W * 4)), ar = step::lds(ou + (uint32_t)(r + RAD) * (W * 4) + 32);
+        float sdv[4];
+        step::step4<false, WD>(w, nullptr, nullptr, al, ar, d[i], b[i], &sq[4 * lane], inj,
+                               warp_int && r >= ri0 && r < ri1, sdx, zs + r, G, K, dn, u1[i], sdv);
+        d[i] = dn;
+        step::sts(ov + (uint32_t)r * (W * 4) + 16, u1[i]);
+        if (!IMG && st_ok && r >= RAD && r < nrel - RAD)
+            *(P4 *)(A.u1_out + sh * A.u1_ss + (zs + r) * NXp + xc) = u1[i];
+    }
+    __syncthreads();
+    // ---- stage B: step 2 at the segment's own planes, on the core
+#pragma unroll
+    for (int i = 0; i < NP; i++) {
+        const int r = py + i * PAR;
+        if (r < RAD || r >= nrel - RAD) continue;
+        const bool inj = inject(e0[i], e1[i], trB, RAD, TX - RAD);
+        P4 w[2 * RAD + 1], dn, un;
+#pragma unroll
+        for (int k = 0; k <= 2 * RAD; k++) w[k] = step::lds(ov + (uint32_t)(r - RAD + k) * (W * 4) + 16);
+        const P4 bl = step::lds(ov + (uint32_t)r * (W * 4)), br = step::lds(ov + (uint32_t)r * (W * 4) + 32);
+        float sdv[4];
+        step::step4<false, WD>(w, nullptr, nullptr, bl, br, d[i], b[i], &sq[4 * lane], inj,
+                               warp_int && r >= ri0 && r < ri1, sdx, zs + r, G, K, dn, un, sdv);
+        if (st_ok) {
+            const int o = (zs + r) * NXp + xc;
+            *(P4 *)(A.u_out + sh * A.u_out_ss + o) = un;
+            *(P4 *)(A.d_out + sh * A.d_out_ss + o) = dn;
+            if (IMG) image_pair(A, sh, o, u1[i], un, sdv);
+        }
+    }
+}
+
 template <int TXT, bool WD, bool IMG = false>
 static void launch2_variant(const GridDev &G, const StencilArgs &A, dim3 grid, cudaStream_t s)
 {
+    if (G.side2) {
+        using S = Stencil2Tile<TXT>;
+        const dim3 tgrid(stencil2_tiles(G) + gather_blocks(A, S::NT), A.nshots);
+        cudaFuncSetAttribute(stencil2_tile_kernel<TXT, WD, IMG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        pdl_launch(stencil2_tile_kernel<TXT, WD, IMG>, tgrid, S::NT, S::SMEM, s, G, A);
+        return;
+    }
     using S = Stencil2Shape<TXT>;
     cudaFuncSetAttribute(stencil2_kernel<TXT, WD, IMG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     pdl_launch(stencil2_kernel<TXT, WD, IMG>, grid, S::NT, S::SMEM, s, G, A);
@@ -384,6 +542,7 @@ int stencil2_blocks_per_sm(const GridDev &G) { return G.tx == 128 ? blocks2_per_
 cudaError_t launch_stencil2(const GridDev &G, const StencilArgs &A, cudaStream_t s)
 {
     if (G.ndim != 2 || G.tti || G.tz2 < 1 || (G.tx != 128 && G.tx != 256)) return cudaErrorInvalidValue;
+    if (G.side2 && G.tz2 > STENCIL2_TILE_Z) return cudaErrorInvalidValue;
     if (A.img && A.wd) return cudaErrorInvalidValue;   // the imaging pair is the adjoint's (u, d) form
     const int cls = A.img ? PROF_STENCIL2_IMG : PROF_STENCIL2;
     cudaEvent_t ev = prof_begin(cls, s);

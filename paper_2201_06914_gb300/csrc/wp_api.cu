@@ -6,6 +6,7 @@
 #include <stdio.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <chrono>
 #include <mutex>
@@ -702,10 +703,17 @@ int choose_tz(const GridDev &G, int nshots)
 // 1601 x 401 grids with 1 to 64 shots: 0.35 + 0.66 f us (throughput, plus half a plane time of
 // unevenness at the end), but 0.36 + 0.5 f us while all blocks are resident and the fields stay
 // in the L2 cache (a lone block's instruction latency, then shared issue slots).  The segment
-// length minimises the product: 3 planes for one shot of 201 x 201 (14 us a launch instead of
-// 27 at 32 planes), 8 for one of 1601 x 401 (17 instead of 25), 32 for 8 shots of it, 61 for 64.
-int choose_tz2(const GridDev &G, int nshots)
+// length minimises the product: 8 planes for one shot of 1601 x 401 (14 us a launch instead of 23
+// at 24 planes), 32 for 8 shots of it, 61 for 64.
+// The other kernel (*side = 1) runs the planes of 8-plane segments side by side, one block a SM at
+// a time: 2.3 us and 2.7 a round of blocks at 128 columns, 3 and 4 at 256, against 4.5 us more than
+// the product for the march (launch, ring and windows).  us a launch, side by side / march: one
+// shot of 150 x 100 4.5 / 7.9, 201 x 201 4.9 / 10.2, 401 x 401 6.5 / 10.6, 4 shots of 201 x 201
+// 10.8 / 13.2, and past the line one shot of 801 x 401 14.3 / 12.5, of 1601 x 401 15.2 / 14.2, 8
+// shots of 201 x 201 18.6 / 14.8.
+int choose_tz2(const GridDev &G, int nshots, int *side)
 {
+    *side = 0;
     if (G.ndim != 2 || G.tti) return 0;
     if (const char *e = getenv("WP_STENCIL2"))
         if (atoi(e) == 0) return 0;
@@ -715,6 +723,10 @@ int choose_tz2(const GridDev &G, int nshots)
     }
     const double cap = (double)device_sm_count() * stencil2_blocks_per_sm(G);
     const double cols = (double)tiles2_x(G) * nshots;
+    GridDev H = G;
+    H.tz2 = STENCIL2_TILE_Z;
+    const double rounds = std::ceil((double)stencil2_tiles(H) * nshots / device_sm_count());
+    const double side_cost = G.tx == 128 ? 2.3 + 2.7 * rounds : 3.0 + 4.0 * rounds;
     const bool in_l2 = 16.0 * (double)G.Np * nshots < 129e6;   // the launch's input and output fields
     int best = G.NZ;
     double cost = 1e300;
@@ -727,6 +739,10 @@ int choose_tz2(const GridDev &G, int nshots)
             best = tz;
         }
     }
+    if (side_cost < cost + 4.5) {
+        *side = 1;
+        return STENCIL2_TILE_Z;
+    }
     return best;
 }
 
@@ -736,7 +752,7 @@ wp_model_s call_model(const wp_model_s *M, const wp_geom *g)
     wp_model_s C = *M;
     const int ns = g ? std::max(1, g->nshots) : 1;
     C.G.tz = choose_tz(C.G, ns);
-    C.G.tz2 = choose_tz2(C.G, ns);
+    C.G.tz2 = choose_tz2(C.G, ns, &C.G.side2);
     return C;
 }
 

@@ -31,6 +31,7 @@ struct GridDev {
     int tx;                // columns of one stencil tile along x (a multiple of 4)
     int tz;                // planes marched by one block (>= 1)
     int tz2;               // planes per two-step segment (0: two-step launches off)
+    int side2;             // 1: the planes of a two-step segment run side by side (small launches)
     float hx, hy, hz;      // grid spacing (m)
     int tti;               // 1: pseudo-acoustic TTI (two fields per shot)
 };
@@ -246,6 +247,7 @@ inline long long stencil_keys(const GridDev &G) { return (long long)stencil_tile
 inline int core2_x(const GridDev &G) { return G.tx - 2 * RAD; }
 inline int tiles2_x(const GridDev &G) { return (G.NXp + core2_x(G) - 1) / core2_x(G); }
 inline int tiles2_z(const GridDev &G) { return (G.NZ + G.tz2 - 1) / G.tz2; }
+constexpr int STENCIL2_TILE_Z = 8;   // segment length where the planes run side by side (G.side2, stencil2.cu)
 // extended segments (one every tz2 planes, tz2 + 8 long) that can hold one plane
 inline int stencil2_seg_reach(const GridDev &G) { return 1 + (2 * RAD + G.tz2 - 1) / G.tz2; }
 inline int stencil2_tiles(const GridDev &G) { return tiles2_x(G) * tiles2_z(G); }

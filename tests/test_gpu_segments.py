@@ -29,6 +29,23 @@ def test_pairs_match_single_steps(nx, nz, off_grid, tz):
         np.testing.assert_array_equal(two[k], one[k], err_msg=k)
 
 
+@pytest.mark.parametrize("tx", ["128", "256"])
+@pytest.mark.parametrize("nx,nz,off_grid", [(104, 31, True), (105, 32, False), (237, 33, True), (17, 3, True)])
+def test_side_by_side_planes_match_single_steps(nx, nz, off_grid, tx):
+    """Small launches at the library's own choice: 8-plane segments whose planes run side by side,
+    grids of a multiple of 8 planes, one less and one more (a last segment of one plane), fewer
+    planes than one block holds, rows on and one past a core of 120 columns.  Bitwise as above."""
+    case = layered_case(ndim=2, nx=nx, nz=nz, nbl=8, nt=37, nshots=2, off_grid=off_grid, zi=0.3, background="const")
+    rng = np.random.default_rng(nx)
+    case.d_obs = rng.standard_normal((2, case.nt, case.rec.shape[1]))
+    Q = rademacher_shots(3, 2, case.nt, 5)
+    one = _run(case, Q, {"WP_STENCIL2": "0", "WP_STENCIL_TX": tx}, Tb=16, ncheck=11)
+    two = _run(case, Q, {"WP_STENCIL2": "1", "WP_STENCIL_TX": tx}, Tb=16, ncheck=11)
+    for k in one:
+        assert np.isfinite(two[k]).all(), k
+        np.testing.assert_array_equal(two[k], one[k], err_msg=k)
+
+
 @pytest.mark.parametrize("nx,ny,nz,tz", [(22, 7, 12, 3), (23, 6, 9, 1), (21, 23, 13, 1000)])
 def test_3d_tile_edges(monkeypatch, nx, ny, nz, tz):
     """3-D tiles of 32 x 16 points: rows and y extents on, one below and one past a tile, marches of
