@@ -704,7 +704,7 @@ int choose_tz(const GridDev &G, int nshots)
 // unevenness at the end), but 0.36 + 0.5 f us while all blocks are resident and the fields stay
 // in the L2 cache (a lone block's instruction latency, then shared issue slots).  The segment
 // length minimises the product: 8 planes for one shot of 1601 x 401 (14 us a launch instead of 23
-// at 24 planes), 32 for 8 shots of it, 61 for 64.
+// at 24 planes), 32 for 8 shots of it, 69 for 64.
 // The other kernel (*side = 1) runs the planes of 8-plane segments side by side, one block a SM at
 // a time: 2.3 us and 2.7 a round of blocks at 128 columns, 3 and 4 at 256, against 4.5 us more than
 // the product for the march (launch, ring and windows).  us a launch, side by side / march: one
