@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "plane_ring.cuh"
 #include "stencil_step.cuh"
 
 namespace wp {
@@ -222,7 +223,8 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, Tti1Shape<TXP, TY>::MI
 #pragma unroll
     for (int k = 0; k < 4; k++) ck[k] = lds2(smem_u32(&coef[k]));
     const bool pad = x + 2 * H > G.NX;   // the points hold row padding: t = 0 there
-    bool failed = false;
+    PlaneRing<NS, LA> pr;
+    auto raise = [&] { if (T.err) atomicExch(T.err, 1); };
     int sc = 0;                          // ring slot of plane z
     uint32_t parity = 0, slot = ring;
     int kz = z0 * PS;
@@ -231,12 +233,12 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, Tti1Shape<TXP, TY>::MI
         for (int ph = 0; ph < U; ph++) {
             const int z = zb + ph;
             if (z >= z1) break;
-            if (tf == 0 && z + LA < z1) {
+            if (tf == 0) {
                 // plane z + LA takes the slot of plane z - (NS - LA), once every warp is past that
                 const int si = sc + LA >= NS ? sc + LA - NS : sc + LA;
-                if (z - z0 >= NS - LA && !failed && !mbar_wait_bounded(&empty[si], parity ^ (sc + LA >= NS ? 0u : 1u)))
-                    failed = true;
-                issue(z + LA, si);
+                pr.refill(z - z0, z1 - z0,
+                          [&] { return mbar_wait_bounded(&empty[si], parity ^ (sc + LA >= NS ? 0u : 1u)); }, raise,
+                          [&] { issue(z + LA, si); });
             }
             __syncwarp();
 #pragma unroll
@@ -245,11 +247,8 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, Tti1Shape<TXP, TY>::MI
                 p0[p] = n0[p];
             }
             ldw(n0, z + RAD + 2 < G.NZ, kz + (RAD + 2) * PS);
-            // a wait that gives up sets the error flag; the march goes on without waiting
-            if (!failed && !mbar_wait_bounded(&full[sc], parity)) {
-                failed = true;
-                if (T.err) atomicExch(T.err, 1);
-            }
+            // a wait that gives up sets the error flag; the march goes on without waiting or issuing
+            pr.await(z - z0, z1 - z0, [&] { return mbar_wait_bounded(&full[sc], parity); }, raise);
             const uint32_t fb = slot + ox;
             f2 q[4 + H];   // x neighbours x-4 .. as aligned pairs
 #pragma unroll
@@ -303,12 +302,8 @@ __global__ void __launch_bounds__(Tti1Shape<TXP, TY>::NT, Tti1Shape<TXP, TY>::MI
 #pragma unroll
             for (int p = 0; p < H; p++) w[k][p] = w[k + U][p];
     }
-    // after a failed wait, let the copies in flight land before the block's memory is reused
-    if (__syncthreads_or(failed) && tid == 0)
-        for (int i = 0; i < NS; i++) {
-            const int n = z1 - z0, cnt = n / NS + (i < n % NS ? 1 : 0);   // planes issued into slot i
-            if (cnt > 0) (void)mbar_wait_bounded(&full[i], (uint32_t)((cnt - 1) & 1));
-        }
+    if (__syncthreads_or(pr.issued) && tf == 0)
+        pr.drain(z1 - z0, [&](int i, uint32_t ph) { (void)mbar_wait_bounded(&full[i], ph); });
     __syncthreads();
 }
 
@@ -707,7 +702,8 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY, ADJ>::NT, TY > 1 ? 4 : 7)
     TtiLayer L = tti_layer(G, sdxy, z0);
     const int zl0 = G.nbl, zl1 = G.nbl + G.nz;   // planes zl0 .. zl1 - 1 lie between the z layers
     const bool pad = x + 2 > G.NX;               // the pair holds row padding: kept at zero
-    bool failed = false;
+    PlaneRing<NS, LA> pr;
+    auto raise = [&] { if (T.err) atomicExch(T.err, 1); };
     int sc = 0;                                  // ring slot of plane z
     uint32_t parity = 0, slot = ring;
     int kz = z0 * PS;
@@ -717,7 +713,8 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY, ADJ>::NT, TY > 1 ? 4 : 7)
             const int z = zb + ph;
             if (z >= z1) break;
             __syncthreads();   // slot of plane z-1 is free again
-            if (z + LA < z1) issue(z + LA, sc + LA >= NS ? sc + LA - NS : sc + LA);
+            pr.refill(z - z0, z1 - z0, [] { return true; }, raise,
+                      [&] { issue(z + LA, sc + LA >= NS ? sc + LA - NS : sc + LA); });
             // own pair of plane z+4 enters the windows; plane z+5 is loaded
             wa[2 * RAD + ph] = step::mul2(qa, q0);
             wb[2 * RAD + ph] = step::mul2(qa, q1);
@@ -738,11 +735,8 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY, ADJ>::NT, TY > 1 ? 4 : 7)
                 prefetch_l2(xf + k7);
             }
             if (z <= zl0 || z >= zl1) L = tti_layer(G, sdxy, z);
-            // a wait that gives up sets the error flag; the march goes on without waiting
-            if (!failed && !mbar_wait_bounded(&full[sc], parity)) {
-                failed = true;
-                if (T.err) atomicExch(T.err, 1);
-            }
+            // a wait that gives up sets the error flag; the march goes on without waiting or issuing
+            pr.await(z - z0, z1 - z0, [&] { return mbar_wait_bounded(&full[sc], parity); }, raise);
             // x parts: five aligned pairs x-4 .. x+5 of t_0, t_1, x_0 and a_x
             f2 p0[5], p1[5], px[5];
 #pragma unroll
@@ -808,12 +802,8 @@ __global__ void __launch_bounds__(Tti2Shape<TXP, TY, ADJ>::NT, TY > 1 ? 4 : 7)
             wx[k] = wx[k + U];
         }
     }
-    // after a failed wait, let the copies in flight land before the block's memory is reused
-    if (__syncthreads_or(failed) && tid == 0)
-        for (int i = 0; i < NS; i++) {
-            const int n = z1 - z0, cnt = n / NS + (i < n % NS ? 1 : 0);   // planes issued into slot i
-            if (cnt > 0) (void)mbar_wait_bounded(&full[i], (uint32_t)((cnt - 1) & 1));
-        }
+    if (__syncthreads_or(pr.issued) && lane == 0)
+        pr.drain(z1 - z0, [&](int i, uint32_t ph) { (void)mbar_wait_bounded(&full[i], ph); });
     __syncthreads();
 }
 
