@@ -13,8 +13,7 @@
 // only multiply the sketch from the right by triangular matrices with positive diagonals).
 #include <cooperative_groups.h>
 
-#include <algorithm>
-
+#include "qr_plan.cuh"
 #include "wp_internal.cuh"
 
 namespace wp {
@@ -48,13 +47,6 @@ cudaError_t launch_transpose(const float *in, long long in_ss, int R, int C, int
     count_launch();
     return cudaGetLastError();
 }
-
-constexpr int QR_THREADS = 512;
-constexpr int QR_MAXR = 512;
-
-// Dynamic shared memory before the CTA's rows: partial dot products of two steps, coefficients,
-// reciprocal squared norms, per-thread partial sums.
-constexpr size_t QR_HEAD = (size_t)(2 * (QR_MAXR + 1) + 2 * QR_MAXR + QR_THREADS) * sizeof(double);
 
 // Thin QR of Y (nt x r per shot, given column-major as Yt[s][i][t]) by CGS2 in FP64.  Writes
 // Q[s][t][i] (row-major, the probe layout) and raises *err (value 3) when a column has no
@@ -187,9 +179,6 @@ cudaError_t launch_cgs2_qr(const float *Yt, int nt, int r, int nshots, double *W
                            cudaStream_t s)
 {
     if (r > QR_MAXR) return cudaErrorInvalidValue;
-    // CTAs per shot: the arithmetic (r^2 nt cycles on one SM) over C, against two reductions of
-    // about 2500 cycles a column (500 within a block), times the rounds in which the device
-    // holds the clusters of all shots (16 shots: clusters of 6 run at once, of 8 in two rounds).
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.y = 1;
@@ -199,35 +188,26 @@ cudaError_t launch_cgs2_qr(const float *Yt, int nt, int r, int nshots, double *W
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(cgs2_qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(cgs2_qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QR_SMEM);
     if (e != cudaSuccess) return e;
-    auto shape = [&](int c, int &rows, bool &in_smem) {
-        rows = (nt + c - 1) / c;
-        const size_t need = QR_HEAD + (size_t)(rows | 1) * r * sizeof(double);
-        in_smem = need <= 227 * 1024;
-        cfg.dynamicSmemBytes = in_smem ? need : QR_HEAD;
+    auto shape = [&](int c, size_t smem) {
+        cfg.dynamicSmemBytes = smem;
         cfg.gridDim = dim3((unsigned)(nshots * c));
         at.val.clusterDim.x = c;
     };
-    int C = 1, rows = nt;
-    bool in_smem = false;
-    double best = 1e300;
-    for (int c = 1; c <= 8; c++) {
-        shape(c, rows, in_smem);
-        int fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, cgs2_qr_kernel, &cfg) != cudaSuccess || fit < 1) {
+    const int C = qr_cluster(nt, r, nshots, [&](int c, bool in_smem) {
+        shape(c, in_smem ? QR_SMEM : QR_HEAD);   // all of an SM's shared memory: one CTA an SM
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, cgs2_qr_kernel, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
-            continue;
+            return 0;
         }
-        const double rounds = (double)((nshots + fit - 1) / fit);
-        const double cost = rounds * ((double)r * r * nt / c + 2.0 * r * (c > 1 ? 2500.0 : 500.0));
-        if (cost < best) {
-            best = cost;
-            C = c;
-        }
-    }
-    shape(C, rows, in_smem);
-    e = cudaLaunchKernelEx(&cfg, cgs2_qr_kernel, Yt, nt, r, rows, in_smem, W, Q, err);
+        return n;
+    });
+    const int rows = (nt + C - 1) / C;
+    const size_t smem = qr_rows_smem(nt, r, C);
+    shape(C, smem ? smem : QR_HEAD);
+    e = cudaLaunchKernelEx(&cfg, cgs2_qr_kernel, Yt, nt, r, rows, smem > 0, W, Q, err);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
