@@ -69,6 +69,12 @@ struct PipeMaps {
     int use;
 };
 
+// Tensor maps of a caller's rows, one per residue of the row number modulo 4 (ROWS).  A type of its
+// own: a launch copies its parameters, 2.3 KB with the ring's maps.
+struct RowMaps {
+    CUtensorMap map[4];
+};
+
 // TMA tensor store / reduce-add of a [64][128] float box from shared memory into P.
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, const void *src, int x, int y, int z)
 {
@@ -210,7 +216,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
 // rows start anywhere too, is read and written by the epilogue's threads.
 template <int RB, int PS, bool ROWS>
 __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeArgs A, const PipePlan PL, int nshots,
-                                                                     const __grid_constant__ PipeMaps TM)
+                                                                     const __grid_constant__ std::conditional_t<ROWS, RowMaps, PipeMaps> TM)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // stays a shared pointer
@@ -269,12 +275,12 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
                 uint8_t *st = stage_ptr(s);
                 if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)((ROWS ? 4 * ROWS_GROUP : rows * 512) + (qlo ? 2 : 1) * img_bytes));
                 __syncwarp();
-                if (ROWS) {
+                if constexpr (ROWS) {
                     // rows G0 .. G0 + 63 of the caller's matrix: sixteen of each residue, from the
                     // first one at or after G0 (rows past the block are masked, past the end zero)
                     if (lane < 4) {
                         const int G0 = (A.ring_ss ? shot * A.cnt : 0) + c * CH;
-                        tma_load_2d(st + lane * ROWS_GROUP, &TM.map[lane >> 1][lane & 1], tile * 128, (G0 - lane + 3) >> 2,
+                        tma_load_2d(st + lane * ROWS_GROUP, &TM.map[lane], tile * 128, (G0 - lane + 3) >> 2,
                                     &full[s]);
                     }
                 } else if (TM.use) {
@@ -496,7 +502,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
             const int shot = item / A.ntiles, tile = item % A.ntiles;
             const uint32_t ab = nacc == 2 ? (j & 1) : 0u, aph = nacc == 2 ? ((j >> 1) & 1) : (j & 1);
             const uint32_t taddr = tmem + ab * ncols + ((uint32_t)(ew * 32) << 16);
-            if (ROWS) {
+            if constexpr (ROWS) {
                 // one point per thread; P of the first 32 probes is read before the wait for the
                 // accumulator, of the next 32 while these are written
                 const long long p = (long long)tile * 128 + e;
@@ -525,37 +531,35 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
                     }
                 }
                 if (bad) break;
-                tc_fence_before();
-                mbar_arrive(&accempty[ab]);
-                continue;
-            }
-            const bool ok = wait_bar(&accfull[ab], aph, &abort_flag);
-            if (epi_any(!ok)) break;
-            tc_fence_after();
+            } else {
+                const bool ok = wait_bar(&accfull[ab], aph, &abort_flag);
+                if (epi_any(!ok)) break;
+                tc_fence_after();
 #pragma unroll
-            for (int c0 = 0; c0 < RB; c0 += PS) {
-                if (c0 < A.r_pad) {
-                    float *stg = stg0 + (size_t)sbuf * PS * 128;
-                    if (e == 0) bulk_wait_read<1>();   // the TMA op that last read this buffer is done
-                    epi_bar();
+                for (int c0 = 0; c0 < RB; c0 += PS) {
+                    if (c0 < A.r_pad) {
+                        float *stg = stg0 + (size_t)sbuf * PS * 128;
+                        if (e == 0) bulk_wait_read<1>();   // the TMA op that last read this buffer is done
+                        epi_bar();
 #pragma unroll
-                    for (int c = c0; c < c0 + PS && c < RB; c += 16) {
-                        if (c < A.r_pad) {
-                            uint32_t r16[16];
-                            tmem_ld16(taddr + (uint32_t)c, r16);
+                        for (int c = c0; c < c0 + PS && c < RB; c += 16) {
+                            if (c < A.r_pad) {
+                                uint32_t r16[16];
+                                tmem_ld16(taddr + (uint32_t)c, r16);
 #pragma unroll
-                            for (int q = 0; q < 16; q++)
-                                stg[(c - c0 + q) * 128 + e] = A.scale * __uint_as_float(r16[q]);
+                                for (int q = 0; q < 16; q++)
+                                    stg[(c - c0 + q) * 128 + e] = A.scale * __uint_as_float(r16[q]);
+                            }
                         }
+                        fence_proxy_async_smem();
+                        epi_bar();
+                        if (e == 0) {
+                            if (A.p_zero) tma_store_3d(&TM.pmap, stg, tile * 128, c0, shot);
+                            else tma_reduce_add_3d(&TM.pmap, stg, tile * 128, c0, shot);
+                            bulk_commit();
+                        }
+                        sbuf ^= 1;
                     }
-                    fence_proxy_async_smem();
-                    epi_bar();
-                    if (e == 0) {
-                        if (A.p_zero) tma_store_3d(&TM.pmap, stg, tile * 128, c0, shot);
-                        else tma_reduce_add_3d(&TM.pmap, stg, tile * 128, c0, shot);
-                        bulk_commit();
-                    }
-                    sbuf ^= 1;
                 }
             }
             tc_fence_before();
@@ -714,7 +718,7 @@ static cudaError_t launch_probe_pipe_slice(const PipeArgs &A, int nshots, cudaSt
 // other: residue rho's map starts at row rho, rounded down to a 16-byte boundary, and its rows are
 // 4 N floats (a multiple of 16 bytes whatever N is) apart; a row ends at its own end, so nothing
 // past the matrix is read.
-static bool rows_maps(const RowsArgs &A, long long nrows, long long x0, long long n, PipeMaps *TM)
+static bool rows_maps(const RowsArgs &A, long long nrows, long long x0, long long n, RowMaps *TM)
 {
     encode_tiled_fn enc = encoder();
     if (!enc || ((uintptr_t)A.a & 15) || nrows > 0x7fffffff) return false;
@@ -725,7 +729,7 @@ static bool rows_maps(const RowsArgs &A, long long nrows, long long x0, long lon
         const cuuint64_t dims[2] = {(cuuint64_t)(n + d), (cuuint64_t)(has ? (nrows - rho + 3) / 4 : 1)};
         const cuuint64_t strides[1] = {(cuuint64_t)A.N * 16};
         const cuuint32_t box[2] = {ROWS_W, 16}, estr[2] = {1, 1};
-        if (enc(&TM->map[rho >> 1][rho & 1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+        if (enc(&TM->map[rho], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
                 (void *)(A.a + x0 + (has ? rho * A.N - d : 0)), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -771,8 +775,7 @@ cudaError_t launch_probe_rows(const RowsArgs &A, int nshots, cudaStream_t s)
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         for (long long x0 = 0; x0 < A.N; x0 += 1LL << 30) {   // a tensor coordinate has 31 bits
-            PipeMaps TM;
-            memset(&TM, 0, sizeof TM);
+            RowMaps TM;
             const long long n = std::min(A.N - x0, 1LL << 30), items = (n + 127) / 128 * nshots;
             if (items >= (1LL << 31) || !rows_maps(A, (long long)A.cnt * (A.a_ss ? nshots : 1), x0, n, &TM))
                 return cudaErrorInvalidValue;
