@@ -578,20 +578,18 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
 
 static int g_num_sms = 0;
 
-// cuTensorMapEncodeTiled from the driver (no link-time dependency on libcuda), or nullptr.
+// cuTensorMapEncodeTiled from the driver (no link-time dependency on libcuda), or nullptr.  Looked up
+// once; first calls from several threads at a time wait for the one that looks it up.
 encode_tiled_fn encoder()
 {
-    static encode_tiled_fn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const encode_tiled_fn fn = [] {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (encode_tiled_fn)p;
-    }
+        const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return ok ? (encode_tiled_fn)p : nullptr;
+    }();
     return fn;
 }
 
