@@ -739,7 +739,8 @@ int choose_tz2(const GridDev &G, int nshots, int *side)
             best = tz;
         }
     }
-    if (side_cost < cost + 4.5) {
+    const char *form = getenv("WP_STENCIL2_SIDE");
+    if (form ? atoi(form) != 0 : side_cost < cost + 4.5) {
         *side = 1;
         return STENCIL2_TILE_Z;
     }
