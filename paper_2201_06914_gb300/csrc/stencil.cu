@@ -16,7 +16,10 @@
 // grid (the Dirichlet exterior costs nothing): a ring holds the u tiles of planes z .. z+4
 // with their x/y halos plus LA planes in flight, a second ring the increment and dt^2/m of
 // the planes being updated.  Internal fields use a row pitch NXp (NX rounded up to 4) so
-// that every float4 is 16-byte aligned; the padding columns stay zero (dt^2/m is zero there).
+// that every float4 is 16-byte aligned.  In the padding columns dt^2/m is zero and the stencil
+// field X (u, or the increment in the (w, d) form) stays zero; Y of the (w, d) form, w, does not:
+// it gathers L d there.  So Y is read at a thread's own points only, where dt^2/m multiplies it,
+// never with halos.
 //
 // Fused into the same launch:
 //   - injection of point sources (forward) or of the receiver residual (adjoint): each

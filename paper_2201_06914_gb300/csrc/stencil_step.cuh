@@ -254,22 +254,5 @@ __device__ __forceinline__ void step4(const P4 *wz, const P4 *wy_p, const P4 *wy
     update4<WD>(wz[RAD], acc, din, bb, sqv, inj, interior, sdx, z, G, K, dn, un, sdv);
 }
 
-// Zero the columns at or beyond the row length (the row padding of the internal layout).
-__device__ __forceinline__ void zero_pad(int xc, int NX, P4 &dn, P4 &un)
-{
-    float d[4], u[4];
-    upk(dn.a, d[0], d[1]);
-    upk(dn.b, d[2], d[3]);
-    upk(un.a, u[0], u[1]);
-    upk(un.b, u[2], u[3]);
-#pragma unroll
-    for (int j = 0; j < 4; j++)
-        if (xc + j >= NX) d[j] = u[j] = 0.f;
-    dn.a = pk(d[0], d[1]);
-    dn.b = pk(d[2], d[3]);
-    un.a = pk(u[0], u[1]);
-    un.b = pk(u[2], u[3]);
-}
-
 }  // namespace step
 }  // namespace wp
