@@ -288,7 +288,7 @@ __global__ void residual_kernel(const float *a, const float *b, float *res, long
 
 // misfit = 1/2 sum of the partials, in a fixed order.  One block of 256 threads: a single thread
 // adding up to 1024 of them took 40 us, most of the call on one shot's record (201 000 values:
-// 48.6 us a call, 7.4 us now).
+// 48.6 us a call, 12 us now: two launches).
 __global__ void finish_misfit_kernel(const double *partials, int nparts, double *misfit)
 {
     pdl_wait();

@@ -1,4 +1,5 @@
-// Pipelined probe accumulation on the tensor cores (Eq. 3).  For every shot and every 128-point tile of the grid:
+// Pipelined probe accumulation on the tensor cores (Eq. 3).  For every shot and every 128-point tile
+// of the grid:
 //   P[i][x] += scale * sum_{t < cnt} A[t][x] * Q[t0 + t][i]
 // where A is read from the time-step ring (forward: u_tt rebuilt from two consecutive
 // stored increments; adjoint: the adjoint wavefield itself) or from a caller's rows of any length
@@ -273,7 +274,9 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
                 const int need = A.cnt - c * CH;
                 const int rows = A.mode ? min(CH + 1, need + 1) : min(CH, need);
                 uint8_t *st = stage_ptr(s);
-                if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)((ROWS ? 4 * ROWS_GROUP : rows * 512) + (qlo ? 2 : 1) * img_bytes));
+                if (lane == 0)
+                    mbar_arrive_expect_tx(&full[s], (uint32_t)((ROWS ? 4 * ROWS_GROUP : rows * 512) +
+                                                               (qlo ? 2 : 1) * img_bytes));
                 __syncwarp();
                 if constexpr (ROWS) {
                     // rows G0 .. G0 + 63 of the caller's matrix: sixteen of each residue, from the
@@ -365,10 +368,11 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) probe_pipe_kernel(const PipeA
         }
     } else if (warp < WEPI) {
         // ---------------- converters ----------------
-        // Up to 64 probes (four stages, a chunk's copy takes 1500 cycles) the converters are two groups of 128 threads (one point each, all 64 steps), one for the
-        // even stages and one for the odd ones, so that one group's shared-memory latencies and
-        // barrier run under the other's work: with all 256 threads on one chunk a chunk took 2000
-        // cycles of mostly waiting.  A group sees every phase of its stages' barriers (a parity
+        // Up to 64 probes (four stages, a chunk's copy takes 1500 cycles) the converters are two
+        // groups of 128 threads (one point each, all 64 steps), one for the even stages and one for
+        // the odd ones, so that one group's shared-memory latencies and barrier run under the
+        // other's work: with all 256 threads on one chunk a chunk took 2000 cycles of mostly
+        // waiting.  A group sees every phase of its stages' barriers (a parity
         // wait cannot tell a phase it skipped from the one before), so chunks go to groups by
         // stage, not by number.  Above, with three stages or fewer, all threads convert every
         // chunk, 32 steps each (256 probes: 5.3 instead of 5.5 ms per 256-step block of 16 shots).
@@ -858,9 +862,9 @@ __global__ void probe_dot_kernel(const float *__restrict__ Pu, bool pu_aligned, 
 }
 
 // Both operands at x pitch NXp with rows `upitch` and `vpitch` floats apart (multiples of 4: the
-// row-aligned layout, or dense rows of a grid whose NX is a multiple of 4): one thread per 4 consecutive points of a row (16-byte loads of
-// both operands; rows of NXp points, a multiple of 4), the same per-point summation order
-// as probe_dot_kernel, so the image is bitwise the same.
+// row-aligned layout, or dense rows of a grid whose NX is a multiple of 4): one thread per 4
+// consecutive points of a row (16-byte loads of both operands; rows of NXp points, a multiple of
+// 4), the same per-point summation order as probe_dot_kernel, so the image is bitwise the same.
 __global__ void probe_dot4_kernel(const float *__restrict__ Pu, long long upitch, const float *__restrict__ Pv,
                                   long long vpitch, long long rows, int NX, int NXp, int r, int nshots, float scale,
                                   float *__restrict__ g)

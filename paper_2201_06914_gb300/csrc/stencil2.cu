@@ -34,9 +34,9 @@
 //     218 and three took 300).
 // Measured per launch of the 1601 x 401 model (padded 1681 x 481): 64 shots 218 us (300 before;
 // 4.75 TB/s of the 20 B per point and shot it must move), 32 shots 121 (167), 16 shots 68 (94.5),
-// 8 shots 41 (57), one shot 15 (33); with the imaging condition, 16 shots: 116 us (150 before,
+// 8 shots 41 (57), one shot 13 (33); with the imaging condition, 16 shots: 116 us (150 before,
 // 130 without the L2 prefetch).  Launches of few blocks run stencil2_tile_kernel (below): one shot
-// of 201 x 201 4.9 us (39 before, 10.2 marching in 3-plane segments), of 401 x 401 6.5 (10.6).
+// of 201 x 201 4.5 us (39 before, 10.0 marching in 3-plane segments), of 401 x 401 5.9 (9.9).
 //
 // Injection uses a CSR table keyed by (tile, plane of the extended segment) that lists
 // every entry inside the extended tile (points in an overlap appear in both tiles);

@@ -21,7 +21,7 @@
 // points; 85 us and 368 for both fields in one thread, 93 us and 582 with two points a thread),
 // pass 2 157 us, 478 per 64 points (201 us, 661: constants re-created at every use, IEEE divisions
 // in a divergent branch, twelve copies a plane issued by one thread).  One step of the padded
-// 336 x 336 x 272 grid: 571 us (737 before), of one shot of 401 x 401 in 2-D: 12.3 us (57).
+// 336 x 336 x 272 grid: 571 us (737 before), of one shot of 401 x 401 in 2-D: 8.9 us (57).
 #include <cuda.h>
 
 #include <algorithm>
@@ -417,8 +417,15 @@ struct TtiLayer {
 };
 // Absorbing layer, s = sigma dt / 2: the update divides by 1 + s.  With rc the correctly
 // rounded reciprocal of c = 1 + s, q = t rc corrected once by its exact remainder, q + (t -
-// c q) rc, is the correctly rounded quotient (Markstein 1990), and t itself where s = 0: three
-// packed operations at every point instead of a branch around IEEE divisions.
+// c q) rc, is the rounded quotient (Markstein 1990; 10^9 random t and c in 1 .. 3 gave the IEEE
+// quotient each time) as long as the remainder does not underflow, and t itself where s = 0: three
+// packed operations at every point instead of a branch around IEEE divisions.  For |t| below about
+// 2^-107 (the foot of a wave front, 30 decades below the wave) the last bit can differ from the IEEE
+// quotient, and an infinite t gives a NaN.  Those bits are enough to give the later rounding another
+// draw: against the IEEE quotient the outputs of a 1000-step 2-D sweep differ by 6e-6, and the
+// errors of either against 64 bits are the same (mean ratio 0.998 over 53 outputs of 27 cases, 2-D
+// and 3-D).  Dividing in the layer gives the former bits and takes 94.3 instead of 84.7 ms on the
+// adjoint of 256 x 256 x 192 and 11.8 instead of 9.4 on the forward of 401 x 401.
 __device__ __forceinline__ TtiLayer tti_layer(const GridDev &G, step::f2 sdxy, int z)
 {
     const step::f2 sd = step::add2(sdxy, step::dup(damp_term(z, G.nz, G.nbl, G.hs0z, G.inv_nbl)));
@@ -519,7 +526,7 @@ __device__ __forceinline__ void tti_update(const TtiArgs &T, const TtiOut &O, lo
 // Pass 2 in 2-D on small launches, as tti_pass1_2d_kernel: one pair of points of both fields in ZP
 // consecutive planes per thread, every load issued before the first use, no shared memory (168
 // registers, 3 blocks a SM).  What bounds it is one latency of the L2 cache and the launch: a step
-// of one shot of 401 x 401 takes 12.3 us, 15.1 with the marching kernel, which has a ring and its
+// of one shot of 401 x 401 takes 8.9 us, 11.8 with the marching kernel, which has a ring and its
 // windows to fill for 3 planes a block (401 x 401 is one wave of this kernel).
 template <int ZP, bool ADJ, bool IMG>
 __global__ void __launch_bounds__(128) tti_pass2_2d_kernel(const GridDev G, const TtiArgs T)
@@ -917,16 +924,33 @@ template <int TX, int TY, int TY1, bool ADJ>
 static cudaError_t tti_passes(const GridDev &G, const TtiArgs &T, cudaStream_t s)
 {
     const int ntx = (G.NX + TX - 1) / TX, nty = (G.NY + TY - 1) / TY, nty1 = (G.NY + TY1 - 1) / TY1;
-    // z segments: a march costs its planes and about five more for the z windows' first planes,
-    // and a plane time grows with the load (choose_segment): 256^3 takes about 30 (within 2 % of
-    // the best of 12 .. 136), one shot of 1601 x 401 6 (24.5 us a step; 36.7 at the former least
-    // of 16).
-    const int tz = choose_segment(G.NZ, (double)ntx * nty * T.nshots, (double)device_sm_count() * (TY > 1 ? 4 : 7), 5.0);
-    const int nseg = (G.NZ + tz - 1) / tz;
-    dim3 grid((unsigned)((long long)ntx * nty * nseg), T.nshots);
     const long long nv = 2LL * T.nshots;
     const float *xf = ADJ ? T.ef_in : T.u_in;
     const long long xss = ADJ ? T.ef_ss : T.u_in_ss;
+    if constexpr (TY == 1) {
+        constexpr int ZP1 = 4, ZP2 = 2;
+        const long long pairs = G.NXp / 2;
+        dim3 grid1((unsigned)((pairs * ((G.NZ + ZP1 - 1) / ZP1) + 127) / 128), T.nshots, 2);
+        pdl_launch(tti_pass1_2d_kernel<ZP1>, grid1, 128, 0, s, G, T);
+        // Up to two waves the direct pass 2 is the faster one (us a step, direct / marching: 201 x 201
+        // 7.7 / 9.6, 401 x 401 8.9 / 11.8, two shots of it 12.3 / 13.5, 801 x 401 12.0 / 13.1; past the
+        // line three shots of 401 x 401 and one of 1201 x 401 were equal within 1 %, 16 shots of
+        // 1601 x 401 251 / 186).  Both give the same bits.
+        const long long blocks = (pairs * ((G.NZ + ZP2 - 1) / ZP2) + 127) / 128;
+        if (blocks * T.nshots <= 2LL * device_sm_count() * pass2_2d_blocks_per_sm()) {
+            dim3 grid2((unsigned)blocks, T.nshots);
+            if (ADJ && T.img) pdl_launch(tti_pass2_2d_kernel<ZP2, true, true>, grid2, 128, 0, s, G, T);
+            else pdl_launch(tti_pass2_2d_kernel<ZP2, ADJ, false>, grid2, 128, 0, s, G, T);
+            return cudaSuccess;
+        }
+    }
+    // z segments: a march costs its planes and about five more for the z windows' first planes,
+    // and a plane time grows with the load (choose_segment): 256^3 takes about 30 (within 2 % of
+    // the best of 12 .. 136), one shot of 1601 x 401 6 (17 us a step; with pass 1 marching too
+    // 24.5, and 36.7 at the former least of 16).
+    const int tz = choose_segment(G.NZ, (double)ntx * nty * T.nshots, (double)device_sm_count() * (TY > 1 ? 4 : 7), 5.0);
+    const int nseg = (G.NZ + tz - 1) / tz;
+    dim3 grid((unsigned)((long long)ntx * nty * nseg), T.nshots);
     if constexpr (TY > 1) {
         using S1 = Tti1Shape<TX, TY1>;
         const long long ass = T.ay - T.ax;   // a_x, a_y and a_z lie one after the other
@@ -939,21 +963,6 @@ static cudaError_t tti_passes(const GridDev &G, const TtiArgs &T, cudaStream_t s
         cudaFuncSetAttribute(tti_pass1_kernel<TX, TY1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S1::SMEM);
         dim3 grid1((unsigned)((long long)ntx * nty1 * nseg), T.nshots);
         pdl_launch(tti_pass1_kernel<TX, TY1>, grid1, S1::NT, S1::SMEM, s, G, T, tz, ntx, nty1, M1);
-    } else {
-        constexpr int ZP1 = 4, ZP2 = 2;
-        const long long pairs = G.NXp / 2;
-        dim3 grid1((unsigned)((pairs * ((G.NZ + ZP1 - 1) / ZP1) + 127) / 128), T.nshots, 2);
-        pdl_launch(tti_pass1_2d_kernel<ZP1>, grid1, 128, 0, s, G, T);
-        // Up to two waves the direct pass 2 is the faster one (400 steps: 201 x 201 4.3 ms instead of
-        // 5.1, 401 x 401 5.25 / 6.1, two shots of it 6.75 / 7.15, 801 x 401 6.3 / 7.1; three shots of
-        // 401 x 401 8.2 / 8.2, 1201 x 401 8.2 / 8.1, 16 shots of 1601 x 401 251 us a step instead of 186)
-        const long long blocks = (pairs * ((G.NZ + ZP2 - 1) / ZP2) + 127) / 128;
-        if (blocks * T.nshots <= 2LL * device_sm_count() * pass2_2d_blocks_per_sm()) {
-            dim3 grid2((unsigned)blocks, T.nshots);
-            if (ADJ && T.img) pdl_launch(tti_pass2_2d_kernel<ZP2, true, true>, grid2, 128, 0, s, G, T);
-            else pdl_launch(tti_pass2_2d_kernel<ZP2, ADJ, false>, grid2, 128, 0, s, G, T);
-            return cudaSuccess;
-        }
     }
 
     using S2 = Tti2Shape<TX, TY, ADJ>;

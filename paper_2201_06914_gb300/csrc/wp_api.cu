@@ -703,14 +703,14 @@ int choose_tz(const GridDev &G, int nshots)
 // 1601 x 401 grids with 1 to 64 shots: 0.35 + 0.66 f us (throughput, plus half a plane time of
 // unevenness at the end), but 0.36 + 0.5 f us while all blocks are resident and the fields stay
 // in the L2 cache (a lone block's instruction latency, then shared issue slots).  The segment
-// length minimises the product: 8 planes for one shot of 1601 x 401 (14 us a launch instead of 23
-// at 24 planes), 32 for 8 shots of it, 69 for 64.
+// length minimises the product: 7 planes for one shot of 1601 x 401 (13 us a launch instead of 23
+// at 24 planes), 31 for 8 shots of it, 69 for 64.
 // The other kernel (*side = 1) runs the planes of 8-plane segments side by side, one block a SM at
 // a time: 2.3 us and 2.7 a round of blocks at 128 columns, 3 and 4 at 256, against 4.5 us more than
 // the product for the march (launch, ring and windows).  us a launch, side by side / march: one
-// shot of 150 x 100 4.5 / 7.9, 201 x 201 4.9 / 10.2, 401 x 401 6.5 / 10.6, 4 shots of 201 x 201
-// 10.8 / 13.2, and past the line one shot of 801 x 401 14.3 / 12.5, of 1601 x 401 15.2 / 14.2, 8
-// shots of 201 x 201 18.6 / 14.8.
+// shot of 150 x 100 4.2 / 7.6, 201 x 201 4.5 / 10.0, 401 x 401 5.9 / 9.9, 4 shots of 201 x 201
+// 10.0 / 12.5, and past the line one shot of 801 x 401 13.4 / 11.9, of 1601 x 401 14.3 / 13.3, 8
+// shots of 201 x 201 17.4 / 13.6 (a sweep's time over its pairs, receivers recorded).
 int choose_tz2(const GridDev &G, int nshots, int *side)
 {
     *side = 0;
