@@ -23,7 +23,8 @@ def test_both_forms_match_single_steps(monkeypatch, nx, nz, off_grid, tx):
     one = _run(case, Q, {"WP_STENCIL2": "0", "WP_STENCIL_TX": tx}, Tb=16, ncheck=11)
     for side in ("0", "1"):
         monkeypatch.setenv("WP_STENCIL2_SIDE", side)
-        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU,
+                                                torch.profiler.ProfilerActivity.CUDA]) as prof:
             two = _run(case, Q, {"WP_STENCIL2": "1", "WP_STENCIL_TX": tx}, Tb=16, ncheck=11)
         ran = {e.key for e in prof.key_averages() if "stencil2" in e.key}
         if ran:   # (no names where the profiler is not available)
