@@ -226,8 +226,8 @@ class Clocks:
 # profiles/pair_and_steps.md) on the default workload: reported only while the
 # kernel's source file still has the hash it was taken on.
 STENCIL_TRAFFIC = {
-    "stencil2.cu": {"sha256_16": "e00c8bbc96b77c59", "shots": 64, "npoints": 1681 * 481,
-                    "bytes_per_launch": 494162944 + 571911424},
+    "stencil2.cu": {"sha256_16": "220b9730f5670cb7", "shots": 64, "npoints": 1681 * 481,
+                    "bytes_per_launch": 493719808 + 572284160},
 }
 
 
@@ -357,12 +357,11 @@ def run_ours(args):
     gm_ms, gm_n = wp.wp_profile_read(1)
     st2_ms, st2_n = wp.wp_profile_read(3)
     wp.wp_profile_enable(False, 0)
-    # Algorithmic bytes of one time step: per shot and point read u^n and the increment,
+    # Algorithmic bytes of a launch.  One step: per shot and point read u^n and the increment,
     # write u^{n+1} and the new increment (16 B); dt^2/m is shared by the shots (4 B per
-    # point once).  A two-step launch processes two steps, so its algorithmic bytes are
-    # twice that; the bytes it must move itself are fewer: it reads u^n and d^n (8 B) and
-    # writes the field the probe contraction needs from the first step (d^{n+1} forward,
-    # v^j adjoint) and u^{n+2}, d^{n+2} (12 B), plus dt^2/m once.
+    # point once).  Two steps: read u^n and d^n (8 B), write the field the probe contraction
+    # needs from the first step (d^{n+1} forward, v^j adjoint) and u^{n+2}, d^{n+2} (12 B),
+    # plus dt^2/m once; st_bytes, what two single steps would move, is reported beside it.
     two = st2_n > 0 and st2_ms >= st1_ms
     st_ms, st_n = (st2_ms, st2_n) if two else (st1_ms, st1_n)
     steps_per_launch = 2 if two else 1
@@ -382,7 +381,7 @@ def run_ours(args):
     except Exception:
         pass
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
-    achieved = st_bytes / st_avg / 1e9
+    achieved = own_bytes / st_avg / 1e9   # bytes the launch must move, not those of two single steps
     gm_gbs = gm_bytes / (gm_ms / 1e3) / 1e9 if gm_ms > 0 else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": achieved / hbm_peak,
@@ -391,11 +390,12 @@ def run_ours(args):
                            "forward/adjoint)") if two else
                           "stencil_kernel<64,1> (2-D, 256-column tiles; forward/adjoint time step)",
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
-                "algorithmic_bytes_per_launch": st_bytes,
-                "algorithmic_unit": "(16 B per point and shot + 4 B per point) per time step",
+                "algorithmic_bytes_per_launch": own_bytes,
+                "algorithmic_unit": (("20" if two else "16") + " B per point and shot + 4 B per point per launch"),
                 "steps_per_launch": steps_per_launch,
-                "kernel_min_bytes_per_launch": own_bytes,
-                "frac_of_kernel_min_bytes": own_bytes / st_avg / 1e9 / hbm_peak,
+                # what as many single-step launches would move, over this launch's time
+                "single_step_bytes_per_launch": st_bytes,
+                "single_step_equivalent_gbs": st_bytes / st_avg / 1e9,
                 "avg_launch_us": st_avg * 1e6, "launches_timed": st_n,
                 "probe_gemm": {"avg_launch_us": gm_ms / max(gm_n, 1) * 1e3, "launches": gm_n,
                                "algorithmic_bytes_per_step": gm_bytes, "achieved_gbs": gm_gbs,
@@ -544,16 +544,18 @@ def run_ours(args):
         img_ms, img_n = (img2_ms, img2_n) if pair_img else (img1_ms, img1_n)
         img_steps = 2 if pair_img else 1
         img_avg = img_ms / max(img_n, 1) / 1e3
-        img_bytes = img_steps * (32.0 * bs + 4.0) * N
+        # a pair reads and writes both fields (16 B), reads three history rows (12 B) and updates the
+        # image (8 B); a single step reads two history rows
+        img_bytes = ((36.0 if pair_img else 32.0) * bs + 4.0) * N
         fwd_avg = fwd_ms / max(fwd_n, 1) / 1e3
-        fwd_bytes = 2 * (16.0 * bs + 4.0) * N
+        fwd_bytes = (20.0 * bs + 4.0) * N
         exact["roofline"] = {
             "kernel": ("stencil2_kernel<64,IMG> (exact adjoint, two steps per launch with g += u_tt v of both fused)"
                        if pair_img else "stencil_kernel<64,1,IMG> (exact adjoint step with g += u_tt v fused)"),
             "bound": "hbm", "avg_launch_us": img_avg * 1e6, "launches": img_n, "steps_per_launch": img_steps,
             "single_step_launches": img1_n if pair_img else 0,
             "algorithmic_bytes_per_launch": img_bytes,
-            "algorithmic_unit": "32 B per point and shot + 4 B per point (dt^2/m) per step",
+            "algorithmic_unit": ("36" if pair_img else "32") + " B per point and shot + 4 B per point per launch",
             "achieved": img_bytes / img_avg / 1e9 if img_n else None, "peak": hbm_peak,
             "frac": (img_bytes / img_avg / 1e9 / hbm_peak) if img_n else None,
             "forward_pairs": {"kernel": "stencil2_kernel<64> (history-writing forward, two steps)",
