@@ -1,7 +1,8 @@
 """Both forms of the two-step launch by name (WP_STENCIL2_SIDE = 1: the planes of 8-plane segments
 side by side, 0: marching), whatever form the cost model would take: every output, the imaging
 variant's among them, is bitwise that of single steps, on launches of a few blocks and of more
-blocks than the device has SMs.  The launch list tells that the form asked for is the one that ran."""
+blocks than the device has SMs.  Where the profiler lists the launches, the form asked for must be the
+one that ran."""
 import numpy as np
 import pytest
 
@@ -27,7 +28,7 @@ def test_both_forms_match_single_steps(monkeypatch, nx, nz, off_grid, tx):
                                                 torch.profiler.ProfilerActivity.CUDA]) as prof:
             two = _run(case, Q, {"WP_STENCIL2": "1", "WP_STENCIL_TX": tx}, Tb=16, ncheck=11)
         ran = {e.key for e in prof.key_averages() if "stencil2" in e.key}
-        if ran:   # (no names where the profiler is not available)
+        if ran:
             assert all(("stencil2_tile_kernel" in k) == (side == "1") for k in ran), ran
         for k in one:
             assert np.isfinite(two[k]).all(), k
